@@ -116,6 +116,8 @@ struct EpiParams {
     float inv_w;
     float w;                // bin width in FP32
     int thr_exact;          // every threshold thr[k] = RN(RN(k w)^2) (computable in-kernel)
+    int no_drop;            // no pair of the problem lies at n_bins or beyond
+    int pos_ok;             // finite coordinates in the range of the branch-free rule
     int n_bins;
     int NW;                 // private bins held per thread (window width)
     int use_window;         // 1: window start derived from per-tile boxes
@@ -224,6 +226,7 @@ struct asd_corr_plan {
     float4 *pos;
     float *thr;
     int thr_exact;             // thr[k] == RN(RN(k w)^2) for every k (see EpiParams)
+    int no_drop, pos_ok;       // see EpiParams
     uint16_t *lut;             // lattice d2 -> bin table (nullptr when d2 can reach kLutMax)
     int n_lut;
     float2 *cs;

@@ -459,7 +459,7 @@ __host__ __device__ inline EpiLayout epi_layout(uint32_t vb, int nb, int nq, int
     L.qacc = take(o, 8u * 2 * (nq > 0 ? nq : 1));
     // fallback bins of pairs outside the private window (FP32, or fixed point)
     L.fb = take(o, (det ? 8u : 4u) * (nb > 0 ? nb : 1));
-    L.colgeo = take(o, 16u * BN);
+    L.colgeo = take(o, 12u * BN);   // x, y, z of the tile's columns, one array each
     L.colpk = take(o, 4u * BN);
     // per-warp row / column boxes, then the boxes of the tile's 32-column chunks (up to 8)
     L.boxred = take(o, 4u * (ew * 12 + 8 * 6));
@@ -579,7 +579,7 @@ enum { BIN_LUT = 0, BIN_THR = 1, BIN_POS = 2 };
 // (FP32 positions, thresholds).
 template <int MODE, int STRIDE>
 __device__ __forceinline__ void bin_chunk(const uint32_t (&g)[32], bool row_ok, int4 ri, float4 rp,
-                                          const float4 *__restrict__ cgeo,
+                                          const float *__restrict__ cg, int BN,
                                           const float *__restrict__ thr,
                                           float *__restrict__ myb, void *__restrict__ fbv,
                                           const BinArgs ba)
@@ -587,14 +587,14 @@ __device__ __forceinline__ void bin_chunk(const uint32_t (&g)[32], bool row_ok, 
     int slot[32];
 #pragma unroll
     for (int k = 0; k < 32; ++k) {
-        const float4 cg = cgeo[k];
+        const float4 cj4 = make_float4(cg[k], cg[BN + k], cg[2 * BN + k], 0.f);
         int b;
         if (MODE == BIN_POS) {
-            b = bin_of_d2_pair(position_d2(rp, cg), ba.inv_w, ba.nb,
+            b = bin_of_d2_pair(position_d2(rp, cj4), ba.inv_w, ba.nb,
                                reinterpret_cast<const float2 *>(thr), ba.err);
         } else {
-            const int4 cj = make_int4(__float_as_int(cg.x), __float_as_int(cg.y),
-                                      __float_as_int(cg.z), 0);
+            const int4 cj = make_int4(__float_as_int(cj4.x), __float_as_int(cj4.y),
+                                      __float_as_int(cj4.z), 0);
             const int d2 = lattice_d2i(ri, cj, ba.Lx, ba.Ly, ba.Lz, ba.periodic);
             if (MODE == BIN_LUT)
                 b = ASD_INB((unsigned)d2 < (unsigned)ba.n_lut, BND_LUT, ba.err)
@@ -625,11 +625,141 @@ __device__ __forceinline__ void bin_chunk(const uint32_t (&g)[32], bool row_ok, 
     }
 }
 
-// Fast lattice form of bin_chunk's first phase (EpiParams::fast): coordinates packed one per byte
-// (x | y<<8 | z<<16), the per-axis minimum image from byte-wise |a - b| and
-// min(d, L - d), d2 from a byte dot product, then the private-bin word offset from the
-// d2 table (LUT, entries pre-scaled by the bin stride) or from the thresholds (THR).
-// Dropped pairs land in the trash row, so no pair takes a branch.
+// ---- branch-free binning: packed FP32 pairs, two columns per instruction ----
+// Issue slots bound this part of the epilogue (two warps per scheduler share the slots of
+// a column's ~50 instructions), so the distance, the guess and the threshold of two
+// columns go through the packed add / mul / fma (one issue for two FP32 results, each
+// rounded as the scalar instruction rounds it).  Measured with the grouped adds below
+// against scalar instructions, two-sided thresholds and one add after the other (64 q in
+// all): 48^3 glass BF16, 2 displacements 139.8 -> 118.3 ms, 32^3 glass split-BF16 22.6 ->
+// 22.0 ms (its other epilogue parts bound it); lattices with the shorter distance below
+// and the grouped adds: 24-sample ensemble 33.7 -> 30.6 ms, 34^3 with K = 444 35.2 -> 26.9.
+__device__ __forceinline__ uint64_t pack2(float a, float b)
+{
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void unpack2(uint64_t v, float &a, float &b)
+{
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b)
+{
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b)
+{
+    uint64_t r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c)
+{
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ float sqrt_guess(float x)
+{
+    float r;
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
+// Constants of the branch-free rule for one tile: 1 / w and w in both halves, the word
+// offset rule off = bin * STRIDE + c0 (c0 takes out the window start and the 2^23 bias of
+// a bin's float form), n_bins, and the trash row of dropped pairs.
+struct FastBin {
+    uint64_t inv2, w2;
+    const float2 *thr2;
+    int nb;
+    uint32_t c0, trash_off;
+};
+constexpr float kBinBase = 8388608.f;          // 2^23: its float holds an integer below
+constexpr uint32_t kBinBaseBits = 0x4B000000u; // 2^23 in the low bits
+
+// Private-bin word offsets of two columns from their squared distances.  The guess is
+// sqrt(d2) / w rounded to nearest, k or k + 1 for an exact bin k (the square root is good
+// to 2^-22, a bin to n_bins <= 4096, so the error is below 1e-2 of a bin), so one threshold
+// decides: bin = guess - (d2 < thr[guess]).  Adding 2^23 rounds without a conversion (like
+// the square root those run on the quarter-rate unit).  EXACT: thr[k] = RN(RN(k w)^2) for
+// every k (the host checks the table), computed; else loaded.  DROP: pairs at n_bins and
+// beyond exist and go to the trash row; otherwise every bin is below n_bins.  Finite
+// coordinates only (the plan checks them; others take the general rule).
+template <bool EXACT, bool DROP, int STRIDE>
+__device__ __forceinline__ void bin2(uint32_t &o0, uint32_t &o1, uint64_t d2, const FastBin &fb)
+{
+    float s0, s1, r0, r1, l0, l1;
+    unpack2(d2, s0, s1);
+    uint64_t x = mul2(pack2(sqrt_guess(s0), sqrt_guess(s1)), fb.inv2);
+    if (DROP) {
+        unpack2(x, r0, r1);
+        x = pack2(fminf(r0, (float)fb.nb), fminf(r1, (float)fb.nb));
+    }
+    const uint64_t g = add2(x, pack2(kBinBase, kBinBase));
+    unpack2(g, r0, r1);
+    if (EXACT) {
+        const uint64_t kw = mul2(add2(g, pack2(-kBinBase, -kBinBase)), fb.w2);
+        unpack2(mul2(kw, kw), l0, l1);
+    } else {
+        l0 = fb.thr2[__float_as_uint(r0) - kBinBaseBits].x;
+        l1 = fb.thr2[__float_as_uint(r1) - kBinBaseBits].x;
+    }
+    const uint32_t b0 = __float_as_uint(r0) - (s0 < l0 ? 1u : 0u);
+    const uint32_t b1 = __float_as_uint(r1) - (s1 < l1 ? 1u : 0u);
+    o0 = b0 * STRIDE + fb.c0;
+    o1 = b1 * STRIDE + fb.c0;
+    if (DROP) {
+        const uint32_t lim = kBinBaseBits + (uint32_t)fb.nb;
+        o0 = b0 < lim ? o0 : fb.trash_off;
+        o1 = b1 < lim ? o1 : fb.trash_off;
+    }
+}
+
+// FP32 positions: the squared distance is position_d2's, fma(dz, dz, fma(dy, dy, dx dx))
+// of FP32 differences, for the row at minus (nx, ny, nz) and columns stored by component.
+template <bool EXACT, bool DROP, int STRIDE>
+__device__ __forceinline__ void pos_offsets(uint32_t (&off)[32], uint64_t nx, uint64_t ny,
+                                            uint64_t nz, const float *__restrict__ cg, int BN,
+                                            const FastBin &fb)
+{
+#pragma unroll
+    for (int k = 0; k < 32; k += 4) {
+        const float4 X = *reinterpret_cast<const float4 *>(cg + k);
+        const float4 Y = *reinterpret_cast<const float4 *>(cg + BN + k);
+        const float4 Z = *reinterpret_cast<const float4 *>(cg + 2 * BN + k);
+        uint64_t d = add2(pack2(X.x, X.y), nx), s = mul2(d, d);
+        d = add2(pack2(Y.x, Y.y), ny);
+        s = fma2(d, d, s);
+        d = add2(pack2(Z.x, Z.y), nz);
+        s = fma2(d, d, s);
+        bin2<EXACT, DROP, STRIDE>(off[k], off[k + 1], s, fb);
+        d = add2(pack2(X.z, X.w), nx);
+        s = mul2(d, d);
+        d = add2(pack2(Y.z, Y.w), ny);
+        s = fma2(d, d, s);
+        d = add2(pack2(Z.z, Z.w), nz);
+        s = fma2(d, d, s);
+        bin2<EXACT, DROP, STRIDE>(off[k + 2], off[k + 3], s, fb);
+    }
+}
+
+// Lattices with byte-sized extents (EpiParams::fast): coordinates packed one per byte
+// (x | y<<8 | z<<16).  Per axis d = |a - b|, e = |L - 2 d| = |d - (L - d)| and the minimum
+// image min(d, L - d) = (L - e) / 2, so one byte dot product of L - e gives 4 d2 (no byte
+// borrows: d < L and e <= L).
+__device__ __forceinline__ uint32_t pk_4d2(uint32_t c, uint32_t rpk, uint32_t Lpk)
+{
+    const uint32_t d = __vabsdiffu4(c, rpk);
+    const uint32_t m = Lpk - __vabsdiffu4(d, Lpk - d);
+    return __dp4a(m, m, 0u);
+}
+
+// Offsets from the d2 -> bin table (entries pre-scaled by the bin stride, the trash row
+// for dropped pairs), or from table thresholds.
 template <bool LUT, int STRIDE>
 __device__ __forceinline__ void pk_offsets(uint32_t (&off)[32], uint32_t rpk, uint32_t Lpk,
                                            const uint4 *__restrict__ cpk,
@@ -644,9 +774,7 @@ __device__ __forceinline__ void pk_offsets(uint32_t (&off)[32], uint32_t rpk, ui
         const uint32_t cc[4] = {c4.x, c4.y, c4.z, c4.w};
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            uint32_t d = __vabsdiffu4(cc[u], rpk);
-            d = __vminu4(d, __vsub4(Lpk, d));
-            const uint32_t d2 = __dp4a(d, d, 0u);
+            const uint32_t d2 = pk_4d2(cc[u], rpk, Lpk) >> 2;
             if (LUT) {
                 off[4 * k4 + u] = ASD_INB(d2 < (uint32_t)n_lut, BND_LUT, err)
                                       ? reinterpret_cast<const uint16_t *>(tab)[d2]
@@ -660,35 +788,29 @@ __device__ __forceinline__ void pk_offsets(uint32_t (&off)[32], uint32_t rpk, ui
     }
 }
 
-// The same bin when every threshold is an exact FP32 square (k w)^2 = RN(RN(k w)^2), as
-// for a power-of-two width (the host checks the whole table): the two thresholds around
-// the first guess are computed instead of loaded.
-__device__ __forceinline__ int bin_of_d2_exact(float d2, float inv_w, float w, int nb)
+// Add 32 values to this thread's private bins, in column order.  One read-modify-write
+// after the other is a chain of shared-memory latencies (the compiler may not move a load
+// above a store that could be to the same bin), so four bins are loaded together and a
+// value whose bin came up earlier in its group takes that sum instead of the loaded one:
+// the same additions in the same order, a quarter of the chain.
+__device__ __forceinline__ void add_private(float *__restrict__ mb, const uint32_t (&off)[32],
+                                            const uint32_t (&g)[32], uint32_t trash_off, int *err)
 {
-    const float r = d2 * rsqrtf(fmaxf(d2, 1e-30f));
-    const int k = min((int)(r * inv_w), nb);
-    const float kw = __fmul_rn((float)k, w), kw1 = __fmul_rn((float)(k + 1), w);
-    const float lo = __fmul_rn(kw, kw), hi = __fmul_rn(kw1, kw1);
-    return k + (d2 >= hi ? 1 : 0) - (d2 < lo ? 1 : 0);
-}
-
-// Fast form of bin_chunk's first phase for FP32 positions, when every pair of the tile
-// falls inside the private window (see the epilogue): the exact bin of each pair from
-// its FP32 d2 and the thresholds (loaded, or computed when EXACT), as a private-bin word
-// offset; dropped pairs go to the trash row, so no pair takes a branch.
-template <int STRIDE, bool EXACT>
-__device__ __forceinline__ void pos_offsets(uint32_t (&off)[32], float4 rp,
-                                            const float4 *__restrict__ cgeo,
-                                            const float2 *__restrict__ thr2, float inv_w,
-                                            float w, int nb, int blo, uint32_t trash_off,
-                                            int *err)
-{
+    (void)trash_off;
+    (void)err;
 #pragma unroll
-    for (int k = 0; k < 32; ++k) {
-        const float d2 = position_d2(rp, cgeo[k]);
-        const int b = EXACT ? bin_of_d2_exact(d2, inv_w, w, nb)
-                            : bin_of_d2_pair(d2, inv_w, nb, thr2, err);
-        off[k] = b < nb ? (uint32_t)((b - blo) * STRIDE) : trash_off;
+    for (int k = 0; k < 32; k += 4) {
+        const uint32_t o0 = off[k], o1 = off[k + 1], o2 = off[k + 2], o3 = off[k + 3];
+        if (!ASD_INB(max(max(o0, o1), max(o2, o3)) <= trash_off, BND_PRIV, err)) continue;
+        float v0 = mb[o0], v1 = mb[o1], v2 = mb[o2], v3 = mb[o3];
+        v0 += __uint_as_float(g[k]);
+        v1 = (o1 == o0 ? v0 : v1) + __uint_as_float(g[k + 1]);
+        v2 = (o2 == o1 ? v1 : o2 == o0 ? v0 : v2) + __uint_as_float(g[k + 2]);
+        v3 = (o3 == o2 ? v2 : o3 == o1 ? v1 : o3 == o0 ? v0 : v3) + __uint_as_float(g[k + 3]);
+        mb[o0] = v0;
+        mb[o1] = v1;
+        mb[o2] = v2;
+        mb[o3] = v3;
     }
 }
 
@@ -1172,7 +1294,7 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) pc_tc_kernel(const __grid_con
         long long *fbi = reinterpret_cast<long long *>(epi + EL.fb);
         long long *cacci = reinterpret_cast<long long *>(epi + EL.cacc);
         long long *qacci = reinterpret_cast<long long *>(epi + EL.qacc);
-        float4 *colgeo = reinterpret_cast<float4 *>(epi + EL.colgeo);
+        float *colgeo = reinterpret_cast<float *>(epi + EL.colgeo);
         uint32_t *colpk = reinterpret_cast<uint32_t *>(epi + EL.colpk);
         float *boxred = reinterpret_cast<float *>(epi + EL.boxred);
         float *chbox = boxred + kEpiWarps * 12;
@@ -1333,13 +1455,16 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) pc_tc_kernel(const __grid_con
                     float4 pj;
                     if (lattice) {
                         const int4 g = E.coords[j];
-                        colgeo[c] = make_float4(__int_as_float(g.x), __int_as_float(g.y),
-                                                __int_as_float(g.z), 0.f);
+                        colgeo[c] = __int_as_float(g.x);
+                        colgeo[BN + c] = __int_as_float(g.y);
+                        colgeo[2 * BN + c] = __int_as_float(g.z);
                         colpk[c] = (uint32_t)g.x | ((uint32_t)g.y << 8) | ((uint32_t)g.z << 16);
                         pj = make_float4((float)g.x, (float)g.y, (float)g.z, 0.f);
                     } else {
                         pj = E.pos[j];
-                        colgeo[c] = pj;
+                        colgeo[c] = pj.x;
+                        colgeo[BN + c] = pj.y;
+                        colgeo[2 * BN + c] = pj.z;
                     }
                     cl[0] = fminf(cl[0], pj.x); ch[0] = fmaxf(ch[0], pj.x);
                     cl[1] = fminf(cl[1], pj.y); ch[1] = fmaxf(ch[1], pj.y);
@@ -1401,7 +1526,7 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) pc_tc_kernel(const __grid_con
                 nwp = E.n_bins;
                 // positions: whether every kept bin of the tile lies inside the private window
                 // [blo, blo + NW), from the largest distance between the two bounding boxes
-                pos_fit = !E.use_window;
+                pos_fit = !E.use_window && E.pos_ok;
                 bhi_tile = E.n_bins - 1;
                 if (E.use_window) {
                     float d2min = 0.f, d2max = 0.f;
@@ -1433,9 +1558,9 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) pc_tc_kernel(const __grid_con
                         bhi_tile = min(E.n_bins - 1,
                                        bin_of_d2_pair(d2max * 1.001f + 1e-30f, E.inv_w, E.n_bins,
                                                       thr2, args.err) + 1);
-                        pos_fit = bhi_tile - blo < E.NW;
+                        pos_fit = E.pos_ok && bhi_tile - blo < E.NW;
                         nwp = bhi_tile - blo + 1;
-                        if (!pos_fit) {
+                        if (!pos_fit && E.pos_ok) {
                             // bins of each 32-column chunk (lane c computes chunk c), then the
                             // first split of the chunks into two windows that together fit
                             int lo_c = 1 << 30, hi_c = -1;
@@ -1561,54 +1686,55 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) pc_tc_kernel(const __grid_con
                             pk_offsets<false, kBinStride>(off, rpk, E.Lpk, cp, thr_s, E.inv_w,
                                                           E.n_bins, trash_off, E.n_lut, args.err);
                         tmem_wait32(g);
-                        if (row_ok) {
-#pragma unroll
-                            for (int k = 0; k < 32; ++k)
-                                if (ASD_INB(off[k] <= trash_off, BND_PRIV, args.err))
-                                    mb[off[k]] += __uint_as_float(g[k]);
-                        }
+                        if (row_ok) add_private(mb, off, g, trash_off, args.err);
                         if (ph) to_bf16(g, tbase + ch * 32, row_ok);
                     }
                 } else if (mode == BIN_POS && pos_fit) {
                     // rows past the range skip the pairs (the TMEM loads stay warp-wide)
                     float *mb = bins + r + kBM * half;
                     const uint32_t trash_off = (uint32_t)E.NW * kBinStride;
-                    const float2 *thr2 = reinterpret_cast<const float2 *>(thr_s);
+                    FastBin fbin = {pack2(E.inv_w, E.inv_w), pack2(E.w, E.w),
+                                    reinterpret_cast<const float2 *>(thr_s), E.n_bins, 0u,
+                                    trash_off};
+                    const uint64_t nx = pack2(-rp.x, -rp.x), ny = pack2(-rp.y, -rp.y),
+                                   nz = pack2(-rp.z, -rp.z);
+                    // whether some pair of the tile may lie at n_bins or beyond
+                    const bool drop = !E.no_drop && (!E.use_window || bhi_tile == E.n_bins - 1);
                     for (int ch = ch0; ch < ch1; ++ch) {
                         // (private row of bin b: b - blo, or b - blo2 + n1 in a second window)
                         const int b0 = !E.use_window ? 0 : ch < split ? blo : blo2 - n1;
                         uint32_t g[32], off[32];
                         tmem_ld32_issue(tbase + ch * 32, g);
-                        if (E.thr_exact)
-                            pos_offsets<kBinStride, true>(off, rp, colgeo + ch * 32, thr2,
-                                                          E.inv_w, E.w, E.n_bins, b0, trash_off,
-                                                          args.err);
+                        const float *cg = colgeo + ch * 32;
+                        fbin.c0 = 0u - (kBinBaseBits + (uint32_t)b0) * (uint32_t)kBinStride;
+                        if (E.thr_exact && !drop)
+                            pos_offsets<true, false, kBinStride>(off, nx, ny, nz, cg, BN, fbin);
+                        else if (E.thr_exact)
+                            pos_offsets<true, true, kBinStride>(off, nx, ny, nz, cg, BN, fbin);
+                        else if (!drop)
+                            pos_offsets<false, false, kBinStride>(off, nx, ny, nz, cg, BN, fbin);
                         else
-                            pos_offsets<kBinStride, false>(off, rp, colgeo + ch * 32, thr2,
-                                                           E.inv_w, E.w, E.n_bins, b0,
-                                                           trash_off, args.err);
+                            pos_offsets<false, true, kBinStride>(off, nx, ny, nz, cg, BN, fbin);
                         tmem_wait32(g);
-                        if (row_ok) {
-#pragma unroll
-                            for (int k = 0; k < 32; ++k)
-                                if (ASD_INB(off[k] <= trash_off, BND_PRIV, args.err))
-                                    mb[off[k]] += __uint_as_float(g[k]);
-                        }
+                        if (row_ok) add_private(mb, off, g, trash_off, args.err);
                         if (ph) to_bf16(g, tbase + ch * 32, row_ok);
                     }
                 } else
                 for (int ch = ch0; ch < ch1; ++ch) {
                     uint32_t g[32];
                     tmem_ld32(tbase + ch * 32, g);
-                    const float4 *cg = colgeo + ch * 32;
+                    const float *cg = colgeo + ch * 32;
                     float *mb = bins + r + kBM * half;
                     void *fbv = fscale != 0.0 ? static_cast<void *>(fbi) : static_cast<void *>(fb);
                     if (mode == BIN_LUT)
-                        bin_chunk<BIN_LUT, kBinStride>(g, row_ok, ri, rp, cg, thr_s, mb, fbv, ba);
+                        bin_chunk<BIN_LUT, kBinStride>(g, row_ok, ri, rp, cg, BN, thr_s, mb, fbv,
+                                                      ba);
                     else if (mode == BIN_THR)
-                        bin_chunk<BIN_THR, kBinStride>(g, row_ok, ri, rp, cg, thr_s, mb, fbv, ba);
+                        bin_chunk<BIN_THR, kBinStride>(g, row_ok, ri, rp, cg, BN, thr_s, mb, fbv,
+                                                      ba);
                     else
-                        bin_chunk<BIN_POS, kBinStride>(g, row_ok, ri, rp, cg, thr_s, mb, fbv, ba);
+                        bin_chunk<BIN_POS, kBinStride>(g, row_ok, ri, rp, cg, BN, thr_s, mb, fbv,
+                                                      ba);
                     if (ph) to_bf16(g, tbase + ch * 32, row_ok);
                 }
             } else if (ph) {

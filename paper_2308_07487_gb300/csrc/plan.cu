@@ -116,6 +116,8 @@ static EpiParams epi_of(const asd_corr_plan *p)
     e.inv_w = p->n_bins > 0 ? (float)(1.0 / p->d.bin_width) : 1.0f;
     e.w = (float)p->d.bin_width;
     e.thr_exact = p->thr_exact;
+    e.no_drop = p->no_drop;
+    e.pos_ok = p->pos_ok;
     e.n_bins = p->n_bins;
     e.NW = p->NW;
     e.use_window = p->use_window;
@@ -540,6 +542,51 @@ int asd_pair_corr_plan_create(const asd_corr_desc *d, asd_corr_plan **out)
         if (max_d2 < kLutMax) p->n_lut = (int)(max_d2 + 1);
     }
 
+    // ---- bin thresholds: (k*w)^2 in FP64, rounded up to FP32 ----
+    std::vector<float> thr((size_t)p->n_bins + 2);
+    thr[0] = 0.f;
+    for (int k = 1; k < p->n_bins + 2; ++k) {
+        double v = ((double)k * d->bin_width) * ((double)k * d->bin_width);
+        float f = (float)v;
+        if ((double)f < v) f = nextafterf(f, INFINITY);
+        thr[k] = f;
+    }
+    // the kernels may compute the thresholds when each equals the FP32 square of the
+    // FP32 product k w (same operations, same rounding, on both sides)
+    p->thr_exact = p->n_bins > 0 && (double)(float)d->bin_width == d->bin_width;
+    for (int k = 0; k < p->n_bins + 2 && p->thr_exact; ++k) {
+        volatile float kw = (float)k * (float)d->bin_width;
+        volatile float sq = kw * kw;
+        p->thr_exact = sq == thr[k];
+    }
+    // whether the branch-free rule holds for the sites (finite squared distances that FP32
+    // holds, widths whose first threshold is a normal number), and whether any pair can
+    // be dropped (largest distance of the bounding box, with room for the FP32 rounding)
+    p->pos_ok = 1;
+    p->no_drop = 0;
+    if (p->n_bins > 0) {
+        double lo[3] = {1e300, 1e300, 1e300}, hi[3] = {-1e300, -1e300, -1e300}, far2 = 0.0;
+        if (d->geometry == ASD_GEOM_POSITIONS) {
+            for (int64_t i = 0; i < p->N; ++i)
+                for (int a = 0; a < 3; ++a) {
+                    const double x = d->pos[3 * i + a];
+                    if (!(fabs(x) <= 1e15)) p->pos_ok = 0;
+                    lo[a] = x < lo[a] ? x : lo[a];
+                    hi[a] = x > hi[a] ? x : hi[a];
+                }
+            for (int a = 0; a < 3; ++a) far2 += (hi[a] - lo[a]) * (hi[a] - lo[a]);
+            far2 *= 1.0 + 1e-5;
+        } else {
+            for (int a = 0; a < 3; ++a) {
+                const double m = d->periodic ? d->L[a] / 2 : d->L[a] - 1;
+                far2 += m * m;
+            }
+        }
+        if (d->bin_width < 1e-12 || d->bin_width > 1e15) p->pos_ok = 0;
+        // (also keeps sqrt(d2) / w far below 2^22, the range of the rounded guess)
+        p->no_drop = p->pos_ok && far2 < (double)thr[p->n_bins];
+    }
+
     // ---- bins: private window per epilogue thread ----
     if (tc) {
         rc = tc_configure(p);
@@ -598,24 +645,7 @@ int asd_pair_corr_plan_create(const asd_corr_desc *d, asd_corr_plan **out)
         if (cudaMemcpy(p->coords, hc.data(), sizeof(int4) * p->N, cudaMemcpyHostToDevice) ||
             cudaMemcpy(p->pos, hp.data(), sizeof(float4) * p->N, cudaMemcpyHostToDevice))
             return fail(ASD_ECUDA);
-        // thresholds (k*w)^2 in FP64, rounded up to FP32
         const int nb = p->n_bins;
-        std::vector<float> thr(nb + 2);
-        thr[0] = 0.f;
-        for (int k = 1; k < nb + 2; ++k) {
-            double v = ((double)k * d->bin_width) * ((double)k * d->bin_width);
-            float f = (float)v;
-            if ((double)f < v) f = nextafterf(f, INFINITY);
-            thr[k] = f;
-        }
-        // the kernels may compute the thresholds when each equals the FP32 square of the
-        // FP32 product k w (same operations, same rounding, on both sides)
-        p->thr_exact = nb > 0 && (double)(float)d->bin_width == d->bin_width;
-        for (int k = 0; k < nb + 2 && p->thr_exact; ++k) {
-            volatile float kw = (float)k * (float)d->bin_width;
-            volatile float sq = kw * kw;
-            p->thr_exact = sq == thr[k];
-        }
         if (cudaMalloc(&p->thr, sizeof(float) * (nb + 2)) != cudaSuccess) {
             cudaGetLastError();
             return fail(ASD_ENOMEM);
