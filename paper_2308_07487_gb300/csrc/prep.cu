@@ -52,16 +52,17 @@ __global__ void means_kernel(const float *__restrict__ traj, int64_t N, int S, i
         for (int a = 0; a < 3; ++a) mean[3 * i + a] = (float)(acc[a] / ((double)S * T0));
 }
 
-// B operand: [N][S*Kseg], 8 consecutive k per thread
+// B operand: [N][S*Kseg], 8 consecutive k per thread; `block` of `blocks` takes a share
 template <int FORM>
-__global__ void prep_b_kernel(const float *__restrict__ traj, int64_t N, int S, int F, int T0,
-                              int Kseg, const float *__restrict__ mean, int center, void *out0,
-                              void *out1)
+__device__ __forceinline__ void prep_b(const float *__restrict__ traj, int64_t N, int S, int F,
+                                       int T0, int Kseg, const float *__restrict__ mean,
+                                       int center, void *out0, void *out1, unsigned block,
+                                       unsigned blocks)
 {
     const int64_t chunks_per_row = (int64_t)S * Kseg / 8;
     const int64_t total = N * chunks_per_row;
-    for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < total;
-         g += (int64_t)gridDim.x * blockDim.x) {
+    for (int64_t g = (int64_t)block * blockDim.x + threadIdx.x; g < total;
+         g += (int64_t)blocks * blockDim.x) {
         const int64_t j = g / chunks_per_row;
         const int64_t kk = (g % chunks_per_row) * 8;
         const int s = (int)(kk / Kseg);
@@ -107,14 +108,15 @@ struct CopyPtrs {
 
 // A operand copies: copy c, row i, elements x..x+V-1 (V = 16 / elem_bytes)
 template <int FORM>
-__global__ void prep_a_kernel(const float *__restrict__ traj, int64_t row_begin, int64_t row_end,
-                              int64_t R, int64_t Rpad, CopyPtrs cp)
+__device__ __forceinline__ void prep_a(const float *__restrict__ traj, int64_t row_begin,
+                                       int64_t row_end, int64_t R, int64_t Rpad,
+                                       const CopyPtrs &cp, unsigned block, unsigned blocks)
 {
     constexpr int V = (FORM == ASD_TF32) ? 4 : 8;  // elements per 16-byte store = copies
     const int64_t chunks = Rpad / V;
     const int64_t total = (row_end - row_begin) * chunks;
-    for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < total;
-         g += (int64_t)gridDim.x * blockDim.x) {
+    for (int64_t g = (int64_t)block * blockDim.x + threadIdx.x; g < total;
+         g += (int64_t)blocks * blockDim.x) {
         const int64_t i = row_begin + g / chunks;
         const int64_t x0 = (g % chunks) * V;
         const float *row = traj + i * R;
@@ -148,6 +150,32 @@ __global__ void prep_a_kernel(const float *__restrict__ traj, int64_t row_begin,
     }
 }
 
+// Both operands in one launch, the first blocks_b blocks the B operand and the rest the A
+// copies (a launch costs a call of a small problem 2 us, as much as its preparation:
+// 16 x 16 sites, T0 = 64, preparation to normalisation 33.1 -> 30.8 us).
+struct PrepArgs {
+    const float *traj;
+    int64_t N;
+    int S, F, T0, Kseg;
+    const float *mean;
+    int center;
+    void *b0, *b1;
+    unsigned blocks_b;
+    int64_t row_begin, row_end, R, Rpad;
+    CopyPtrs cp;
+};
+
+template <int FORM>
+__global__ void __launch_bounds__(256) prep_kernel(const __grid_constant__ PrepArgs a)
+{
+    if (blockIdx.x < a.blocks_b)
+        prep_b<FORM>(a.traj, a.N, a.S, a.F, a.T0, a.Kseg, a.mean, a.center, a.b0, a.b1,
+                     blockIdx.x, a.blocks_b);
+    else if constexpr (FORM != ASD_FP32)
+        prep_a<FORM>(a.traj, a.row_begin, a.row_end, a.R, a.Rpad, a.cp,
+                     blockIdx.x - a.blocks_b, gridDim.x - a.blocks_b);
+}
+
 unsigned grid_for(int64_t work, int sm_count)
 {
     int64_t b = (work + 255) / 256;
@@ -165,41 +193,34 @@ int launch_prep(asd_corr_plan *p, const float *traj, int64_t row_begin, int64_t 
         means_kernel<<<(unsigned)((p->N + 7) / 8), 256, 0, s>>>(traj, p->N, S, F, T0, p->meanB);
         ASD_CUDA_TRY(cudaGetLastError());
     }
-    const int64_t bwork = p->N * p->Kb / 8;
-    const unsigned gb = grid_for(bwork, p->sm_count);
-    switch (p->prec) {
-    case ASD_FP32:
-        prep_b_kernel<ASD_FP32><<<gb, 256, 0, s>>>(traj, p->N, S, F, T0, (int)p->Kseg, p->meanB,
-                                                   p->center, p->Bf32, nullptr);
-        break;
-    case ASD_TF32:
-        prep_b_kernel<ASD_TF32><<<gb, 256, 0, s>>>(traj, p->N, S, F, T0, (int)p->Kseg, p->meanB,
-                                                   p->center, p->B[0], nullptr);
-        break;
-    case ASD_BF16:
-        prep_b_kernel<ASD_BF16><<<gb, 256, 0, s>>>(traj, p->N, S, F, T0, (int)p->Kseg, p->meanB,
-                                                   p->center, p->B[0], nullptr);
-        break;
-    default:
-        prep_b_kernel<ASD_SPLIT_BF16><<<gb, 256, 0, s>>>(traj, p->N, S, F, T0, (int)p->Kseg,
-                                                         p->meanB, p->center, p->B[0], p->B[1]);
-        break;
-    }
-    ASD_CUDA_TRY(cudaGetLastError());
-    if (!p->tc) return ASD_OK;
-    CopyPtrs cp{};
+    PrepArgs a{};
+    a.traj = traj;
+    a.N = p->N;
+    a.S = S;
+    a.F = F;
+    a.T0 = T0;
+    a.Kseg = (int)p->Kseg;
+    a.mean = p->meanB;
+    a.center = p->center;
+    a.b0 = p->tc ? p->B[0] : p->Bf32;
+    a.b1 = p->B[1];
+    a.blocks_b = grid_for(p->N * p->Kb / 8, p->sm_count);
+    a.row_begin = row_begin;
+    a.row_end = row_end;
+    a.R = p->R;
+    a.Rpad = p->Rpad;
     for (int pl = 0; pl < p->n_planes; ++pl)
-        for (int c = 0; c < p->n_copies; ++c) cp.p[pl][c] = p->A[pl][c];
-    const int V = p->prec == ASD_TF32 ? 4 : 8;
-    const int64_t awork = (row_end - row_begin) * (p->Rpad / V);
-    const unsigned ga = grid_for(awork, p->sm_count);
-    if (p->prec == ASD_TF32)
-        prep_a_kernel<ASD_TF32><<<ga, 256, 0, s>>>(traj, row_begin, row_end, p->R, p->Rpad, cp);
-    else if (p->prec == ASD_BF16)
-        prep_a_kernel<ASD_BF16><<<ga, 256, 0, s>>>(traj, row_begin, row_end, p->R, p->Rpad, cp);
-    else
-        prep_a_kernel<ASD_SPLIT_BF16><<<ga, 256, 0, s>>>(traj, row_begin, row_end, p->R, p->Rpad,
-                                                         cp);
+        for (int c = 0; c < p->n_copies; ++c) a.cp.p[pl][c] = p->A[pl][c];
+    unsigned blocks = a.blocks_b;
+    if (p->tc && row_end > row_begin)
+        blocks += grid_for((row_end - row_begin) * (p->Rpad / (p->prec == ASD_TF32 ? 4 : 8)),
+                           p->sm_count);
+    switch (p->prec) {
+    case ASD_FP32: prep_kernel<ASD_FP32><<<blocks, 256, 0, s>>>(a); break;
+    case ASD_TF32: prep_kernel<ASD_TF32><<<blocks, 256, 0, s>>>(a); break;
+    case ASD_BF16: prep_kernel<ASD_BF16><<<blocks, 256, 0, s>>>(a); break;
+    default: prep_kernel<ASD_SPLIT_BF16><<<blocks, 256, 0, s>>>(a); break;
+    }
     ASD_CUDA_TRY(cudaGetLastError());
     return ASD_OK;
 }
