@@ -134,6 +134,8 @@ struct EpiParams {
     int npass;              // passes of kPhaseQ q-vectors (0 without phase weights)
     int q_parts;            // 1: cosine part of the phase sum; 2: cosine and sine parts
     const float2 *cs;       // [N][nq_pad] (cos, sin)(q.r_i)
+    const float2 *csT;      // the same by q: [nq_pad][cs_ld] (tensor forms)
+    int64_t cs_ld;          // row length of csT
     double *C_sum;          // [n_t][n_bins]
     double *Sq_sum;         // [n_t][n_q]
     // deterministic mode: fixed-point sums [n_t][n_bins] and [n_t][n_q][q_parts] and the
@@ -143,14 +145,8 @@ struct EpiParams {
     const double *fix_scale;
 };
 
-// One problem of the (possibly batched) tensor-core launch.
-struct TcProblem {
-    CUtensorMap mapA[2][kMaxCopies];  // [plane][copy]
-    CUtensorMap mapB[2];              // [plane]
-    CUtensorMap mapW[2];              // phase column weights [plane]: rows (pass, output),
-                                      // columns = sites (BF16 hi / lo)
-    int64_t tile_begin;               // first flattened work item of this problem
-    int64_t n_tiles;                  // work items: n_t * tiles_m * tiles_n
+// Sizes of one problem that the roles of the kernel walk by.
+struct TcDims {
     int N;                            // columns (sites)
     int row_begin, row_end;
     int tiles_m, tiles_n;
@@ -162,6 +158,18 @@ struct TcProblem {
     int n_copies;                     // shifted copies (8 for BF16, 4 for TF32)
     int group_m;                      // raster group height (row tiles)
     int k_chunks;                     // partial accumulators along K per tile
+    int npass;                        // passes of kPhaseQ q-vectors
+};
+
+// One problem of the (possibly batched) tensor-core launch.
+struct TcProblem {
+    CUtensorMap mapA[2][kMaxCopies];  // [plane][copy]
+    CUtensorMap mapB[2];              // [plane]
+    CUtensorMap mapW[2];              // phase column weights [plane]: rows (pass, output),
+                                      // columns = sites (BF16 hi / lo)
+    int64_t tile_begin;               // first flattened work item of this problem
+    int64_t n_tiles;                  // work items: n_t * tiles_m * tiles_n
+    TcDims dims;
     EpiParams epi;
 };
 
@@ -180,12 +188,14 @@ struct TcOverride {
 struct TcLaunchArgs {
     const TcProblem *probs;
     int n_probs;
+    TcDims one;            // n_probs = 1: its sizes (kernel parameters need no memory access)
     int64_t total_tiles;
     TcOverride ov;
     int stages;
     uint32_t VB;           // bytes of the per-problem epilogue region (largest problem)
-    unsigned long long *counter;  // dynamic schedule: work-item counter (zero at launch), or null
-    int NB, NQ;            // epilogue shared-memory layout maxima
+    unsigned long long *counter;  // dynamic schedule: work-item counter and finished CTAs (both
+                                  // zero between launches), or null
+    int NB, NQ;            // epilogue shared-memory layout maxima (n_bins, n_q * q_parts)
     int det;               // 1: some problem sums in fixed point (fallback bins 8 bytes)
     int *err;
 };
@@ -229,11 +239,11 @@ struct asd_corr_plan {
     int no_drop, pos_ok;       // see EpiParams
     uint16_t *lut;             // lattice d2 -> bin table (nullptr when d2 can reach kLutMax)
     int n_lut;
-    float2 *cs;
+    float2 *cs, *csT;          // (cos, sin)(q.r_i) by site; by q (tensor forms)
     void *W;                   // phase column weights [2 planes][npass * 128][Wld] BF16
     int64_t Wld;               // row length of W (N rounded up to 8)
     double *sqF;               // separable phase form: transforms [2 n_q][S*3F] (n_q > 0)
-    unsigned long long *counter;  // work-item counter of the dynamic schedule
+    unsigned long long *counter;  // [2]: the dynamic schedule's work items claimed, CTAs done
     int q_parts;               // 1 + desc.phase_sine: values per (t, q) in Sq_sum
     int tiles_m_all, tiles_n;
     int use_window;
@@ -272,7 +282,8 @@ int launch_simt(asd_corr_plan *p, const float *traj, int64_t row_begin, int64_t 
                 int t_begin, int t_end, double *C_sum, double *Sq_sum, cudaStream_t s);
 // pc_tc.cu
 int tc_configure(asd_corr_plan *p);    // stages / smem for the plan's form
-int launch_tc(const TcProblem *d_probs, int n_probs, int64_t total_tiles, TcOverride ov, int prec,
+int launch_tc(const TcProblem *d_probs, int n_probs, const TcDims &one, int64_t total_tiles,
+              TcOverride ov, int prec,
               int BN, int swizzle_bytes, int stages, size_t smem, uint32_t var_bytes,
               int max_nb, int max_nq, int ew, int det, int cg, int sm_count,
               unsigned long long *counter, cudaStream_t s);

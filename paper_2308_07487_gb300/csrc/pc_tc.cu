@@ -33,7 +33,7 @@ static int configure_once(asd_corr_plan *p, size_t cap, size_t stage_bytes)
     int NW = p->n_bins;
     p->use_window = 0;
     auto epi = [&](int nw) {
-        return tc_epilogue_smem(nw, p->n_bins, p->n_q, p->BN, p->n_lut, p->EW, p->d.deterministic);
+        return tc_epilogue_smem(nw, p->n_bins, p->n_q * p->q_parts, p->BN, p->n_lut, p->EW, p->d.deterministic);
     };
     for (int min_st = 3; min_st >= 2; --min_st) {
         NW = p->n_bins;
@@ -74,7 +74,7 @@ int tc_configure(asd_corr_plan *p)
     if (st > 8) st = 8;
     if (p->d.stages > 0 && p->d.stages < st) st = p->d.stages;
     p->stages = st;
-    p->smem_bytes = tc_epilogue_smem(p->NW, p->n_bins, p->n_q, p->BN, p->n_lut, p->EW,
+    p->smem_bytes = tc_epilogue_smem(p->NW, p->n_bins, p->n_q * p->q_parts, p->BN, p->n_lut, p->EW,
                                      p->d.deterministic) +
                     (size_t)p->stages * stage_bytes + 2048;
     // more than half of the SM's shared memory: never two CTAs (and TMEM owners) per SM
@@ -82,7 +82,8 @@ int tc_configure(asd_corr_plan *p)
     return ASD_OK;
 }
 
-int launch_tc(const TcProblem *d_probs, int n_probs, int64_t total_tiles, TcOverride ov, int prec,
+int launch_tc(const TcProblem *d_probs, int n_probs, const TcDims &one, int64_t total_tiles,
+              TcOverride ov, int prec,
               int BN, int swizzle_bytes, int stages, size_t smem, uint32_t var_bytes_,
               int max_nb, int max_nq, int ew, int det, int cg, int sm_count,
               unsigned long long *counter, cudaStream_t s)
@@ -91,13 +92,14 @@ int launch_tc(const TcProblem *d_probs, int n_probs, int64_t total_tiles, TcOver
     LaunchArgs a{};
     a.probs = d_probs;
     a.n_probs = n_probs;
+    a.one = one;
     a.total_tiles = total_tiles;
     a.ov = ov;
     a.stages = stages;
     a.VB = var_bytes_;
-    // dynamic schedule: the counter starts at zero for every launch (stream-ordered)
+    // dynamic schedule: the counter (and the count of finished CTAs behind it) is zero at
+    // every launch; the launch's last CTA leaves it so
     a.counter = counter;
-    if (a.counter) ASD_CUDA_TRY(cudaMemsetAsync(a.counter, 0, sizeof(unsigned long long), s));
     a.NB = max_nb;
     a.NQ = max_nq;
     a.det = det;

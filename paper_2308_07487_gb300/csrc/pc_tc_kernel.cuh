@@ -10,6 +10,10 @@
 //   warp 1      allocates TMEM and, from one thread, issues tcgen05.mma into one of two
 //               128 x BN FP32 accumulators in tensor memory (double buffered), committing
 //               each stage back to the ring and each finished work item to the epilogue;
+//   then one    geometry: one tile ahead of the epilogue, loads the tile's column geometry
+//               into one of two shared-memory buffers and finds its bin window(s);
+//   then four   (tiles of at most 192 columns) read the phase product out of TMEM, one warp
+//               per lane quarter;
 //   warps 2..   epilogue (EW = 4 or 8 warps): reads the accumulator from TMEM and
 //               reduces it -- per-thread private FP32 bins in shared memory
 //               (conflict-free [bin][row] layout), phase weights from per-site cos/sin
@@ -41,7 +45,8 @@ namespace asd {
 namespace {
 
 // Epilogue warps EW (template parameter): 4 (one per TMEM lane quarter, all columns) or
-// 8 (two per quarter, half the columns each).  Threads = TMA warp + MMA warp + EW warps.
+// 8 (two per quarter, half the columns each).  Threads = TMA warp + MMA warp + EW warps +
+// geometry warp + phase read-out warps.
 constexpr int kMaxEpiWarps = 8;
 constexpr unsigned long long kTimeoutNs = 4000000000ull;
 // TMEM: 512 columns per CTA (one CTA per SM): two BN-column accumulators, then (phase
@@ -54,7 +59,20 @@ constexpr uint32_t kWBytes = 128u * 128u;     // one plane of a W stage: 128 row
 // claims each item from a global counter, so the items in flight across the grid stay
 // together whatever each item costs (L2 reuse of A / B panels, no drift, balanced tail);
 // the static schedule takes, in round k of n CTAs, item k n + (cid + k) mod n.
+//
+// A slot holds the decoded sub-item, so only the TMA thread decodes (its 64-bit divisions
+// and descriptor reads cost every epilogue thread 0.7 to 2.1 thousand cycles per sub-item
+// before), and it decodes the next item in the middle of the current one's K blocks, its
+// claim from the counter made an item earlier still.
 constexpr int kWQ = 4;
+struct __align__(16) WorkSlot {
+    int p;          // problem, -1: no work left
+    int t, m0, n0;  // displacement, first row and column of the tile
+    int row_end;
+    int kci;        // K chunk of the tile, 0: first
+    int last;       // 1: the tile's last chunk
+    int nk;         // K blocks of the chunk
+};
 // Private bins are a [bin][128 * EW/4] array: epilogue thread (row r, column half h)
 // only ever touches column r + 128 h, i.e. bank r mod 32, so the per-pair accumulation
 // is free of bank conflicts whatever the bins of the 32 lanes are (with an odd stride,
@@ -282,27 +300,21 @@ __device__ __forceinline__ void tc_mma_ts(uint32_t d, uint32_t a_tmem, uint64_t 
             "r"(a_tmem), "l"(b), "r"(idesc), "r"(acc));
 }
 
-// 32 lanes x 16 consecutive 32-bit columns (this thread's lane), and its wait, tied to the
+// 32 lanes x 8 consecutive 32-bit columns (this thread's lane), and its wait, tied to the
 // registers.
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16])
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8])
 {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, "
-        "%11, %12, %13, %14, %15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-          "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]),
-          "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr));
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]),
+                   "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr));
 }
-__device__ __forceinline__ void tmem_wait16x2(uint32_t (&a)[16], uint32_t (&b)[16])
+__device__ __forceinline__ void tmem_wait8x2(uint32_t (&a)[8], uint32_t (&b)[8])
 {
     asm volatile("tcgen05.wait::ld.sync.aligned;"
                  : "+r"(a[0]), "+r"(a[1]), "+r"(a[2]), "+r"(a[3]), "+r"(a[4]), "+r"(a[5]),
-                   "+r"(a[6]), "+r"(a[7]), "+r"(a[8]), "+r"(a[9]), "+r"(a[10]), "+r"(a[11]),
-                   "+r"(a[12]), "+r"(a[13]), "+r"(a[14]), "+r"(a[15]), "+r"(b[0]), "+r"(b[1]),
-                   "+r"(b[2]), "+r"(b[3]), "+r"(b[4]), "+r"(b[5]), "+r"(b[6]), "+r"(b[7]),
-                   "+r"(b[8]), "+r"(b[9]), "+r"(b[10]), "+r"(b[11]), "+r"(b[12]), "+r"(b[13]),
-                   "+r"(b[14]), "+r"(b[15])
+                   "+r"(a[6]), "+r"(a[7]), "+r"(b[0]), "+r"(b[1]), "+r"(b[2]), "+r"(b[3]),
+                   "+r"(b[4]), "+r"(b[5]), "+r"(b[6]), "+r"(b[7])
                  :
                  : "memory");
 }
@@ -420,8 +432,18 @@ __host__ __device__ constexpr uint32_t idesc(bool tf32, int N, int M = kBM)
 // ------------------------------------------------------------------------------------
 // shared-memory layout of the epilogue region
 // ------------------------------------------------------------------------------------
+// Bin window(s) of a tile.  One window: private row k holds bin blo + k.  Positions whose
+// columns join two far-apart groups of sites may take two: rows [0, n1) for bins blo + k
+// (column chunks before `split`), rows [n1, nwp) for bins blo2 + k - n1.
+struct TileWindow {
+    int blo, blo2, n1, nwp, split;
+    int bhi;       // largest bin the tile can keep (positions)
+    int fit;       // positions: every kept bin of the tile is in the window(s)
+    int pad;
+};
+
 struct EpiLayout {
-    uint32_t cacc, qacc, fb, colgeo, colpk, boxred, var, total;
+    uint32_t cacc, qacc, fb, geo, win, par, var, total;
 };
 
 __host__ __device__ inline uint32_t take(uint32_t &o, uint32_t bytes)
@@ -455,90 +477,88 @@ __host__ __device__ inline EpiLayout epi_layout(uint32_t vb, int nb, int nq, int
     uint32_t o = 0;
     // per-CTA bin sums (FP64, or 64-bit fixed point in the deterministic mode)
     L.cacc = take(o, 8u * (nb > 0 ? nb : 1));
-    // phase sums per q: (cosine, sine) parts (FP64 or fixed point)
-    L.qacc = take(o, 8u * 2 * (nq > 0 ? nq : 1));
+    // phase sums per TMEM lane quarter and (q, part), nq = n_q * parts (FP64 or fixed point);
+    // each quarter's sums belong to its read-out warp
+    L.qacc = take(o, 8u * 4 * (nq > 0 ? nq : 1));
     // fallback bins of pairs outside the private window (FP32, or fixed point)
     L.fb = take(o, (det ? 8u : 4u) * (nb > 0 ? nb : 1));
-    L.colgeo = take(o, 12u * BN);   // x, y, z of the tile's columns, one array each
-    L.colpk = take(o, 4u * BN);
-    // per-warp row / column boxes, then the boxes of the tile's 32-column chunks (up to 8)
-    L.boxred = take(o, 4u * (ew * 12 + 8 * 6));
+    // two tiles' column geometry (x, y, z arrays, or one array of packed coordinates) and bin
+    // windows, filled by the geometry warp
+    L.geo = take(o, 2u * 12u * BN);
+    L.win = take(o, 2u * (uint32_t)sizeof(TileWindow));
+    // the current problem's parameters (global memory is several hundred cycles away while
+    // the operand streams run)
+    L.par = take(o, (uint32_t)sizeof(EpiParams) + 16u);
     L.var = take(o, vb);
     L.total = (o + 1023u) & ~1023u;
     return L;
 }
 
-struct TileInfo {
-    int p, t, m0, n0, row_end;
-    int kg0, kg1;  // K blocks [kg0, kg1) of the S * nkb blocks of a full row
-};
-
-// Work item `tau` -> (problem, t, row tile, column tile), sub-item c -> its K chunk c.  K
-// chunks split the contraction so that each partial accumulator starts from zero.
-// Per-role walk over the work list.  A role visits its work items in increasing order,
-// so the problem of the next item is found by stepping forward from the current one, and
-// the fields that decoding needs stay in registers until the problem changes (a batched
-// launch would otherwise repeat a search over the descriptors in global memory per item).
+// Per-role walk over the work list: the fields that decoding needs stay in registers until
+// the problem changes (a batched launch would otherwise search the descriptors per item).
 struct WorkCursor {
     int p = -1;
     int64_t begin = 0, end = 0;  // flattened work items [begin, end) belong to problem p
     int tiles_m, tiles_n, kch, G, nk, row_begin, row_end, t_begin;
+    int nkb, F3, n_copies, Kseg, npass;
     int64_t per_t;
 };
 
-// A work item is one (problem, displacement, row tile, column tile); its K chunks are
-// consecutive sub-items on the same CTA (they share the tile's geometry and private
-// bins).  decode(tau, c) gives chunk c of work item tau.  Row tiles are row_step rows
-// (256 for a CTA pair, whose second CTA takes rows row_off = 128 on).
+// a / b of non-negative numbers, in 32 bits where they fit (a 64-bit division takes about
+// a hundred instructions).
+__device__ __forceinline__ int64_t div_small(int64_t a, int64_t b)
+{
+    if (((a | b) >> 32) == 0) return (int64_t)((uint32_t)a / (uint32_t)b);
+    return a / b;
+}
+
+// A tile of the work list.
+struct TileInfo {
+    int t, m0, n0;
+};
+
+// Work item tau = one (problem, displacement, row tile, column tile) in grouped raster order;
+// its K chunks are consecutive sub-items on the same CTA (they share the tile's geometry and
+// private bins).  Row tiles are row_step rows (256 for a CTA pair, whose second CTA takes
+// rows row_off = 128 on).
 __device__ __forceinline__ TileInfo decode(WorkCursor &cu, const TcProblem *__restrict__ probs,
-                                           int n_probs, const TcOverride &ov, int64_t tau,
-                                           int c, int BN, int row_step = kBM, int row_off = 0)
+                                           int n_probs, const TcDims &one, const TcOverride &ov,
+                                           int64_t tau, int BN, int row_step, int row_off)
 {
     if (cu.p < 0 || tau >= cu.end) {
         int p = cu.p < 0 ? 0 : cu.p;
-        if (n_probs > 1) {
-            if (cu.p < 0) {
-                int lo = 0, hi = n_probs - 1;
-                while (lo < hi) {
-                    int mid = (lo + hi + 1) >> 1;
-                    if (probs[mid].tile_begin <= tau) lo = mid;
-                    else hi = mid - 1;
-                }
-                p = lo;
-            } else {
-                while (p + 1 < n_probs && probs[p + 1].tile_begin <= tau) ++p;
-            }
-        }
-        const TcProblem &P = probs[p];
+        while (p + 1 < n_probs && probs[p + 1].tile_begin <= tau) ++p;
+        const TcDims P = n_probs == 1 ? one : probs[p].dims;
         cu.p = p;
         const int tiles_m = ov.active ? ov.tiles_m : P.tiles_m;
-        cu.begin = ov.active ? 0 : P.tile_begin;
-        cu.end = cu.begin + (ov.active ? ov.n_tiles : P.n_tiles);
+        cu.begin = ov.active ? 0 : probs[p].tile_begin;
+        cu.end = cu.begin + (ov.active ? ov.n_tiles : probs[p].n_tiles);
         cu.tiles_m = tiles_m;
         cu.tiles_n = P.tiles_n;
         cu.kch = P.k_chunks;
         cu.G = max(1, P.group_m);
+        cu.nkb = P.nkb;
         cu.nk = P.S * P.nkb;
+        cu.F3 = P.F3;
+        cu.n_copies = P.n_copies;
+        cu.Kseg = P.Kseg;
+        cu.npass = P.npass;
         cu.row_begin = ov.active ? ov.row_begin : P.row_begin;
         cu.row_end = ov.active ? ov.row_end : P.row_end;
         cu.t_begin = ov.active ? ov.t_begin : 0;
         cu.per_t = (int64_t)cu.tiles_m * cu.tiles_n;
     }
     const int64_t l = tau - cu.begin;
-    TileInfo ti;
-    ti.p = cu.p;
-    ti.t = cu.t_begin + (int)(l / cu.per_t);
-    const int kc = c;
-    const int64_t rem = l % cu.per_t;
+    const int64_t t = div_small(l, cu.per_t), rem = l - t * cu.per_t;
     const int64_t gspan = (int64_t)cu.G * cu.tiles_n;
-    const int first_m = (int)(rem / gspan) * cu.G;
+    const int64_t grp = div_small(rem, gspan), r2 = rem - grp * gspan;
+    const int first_m = (int)grp * cu.G;
     const int gsz = min(cu.G, cu.tiles_m - first_m);
-    const int64_t r2 = rem % gspan;
-    ti.m0 = cu.row_begin + (first_m + (int)(r2 % gsz)) * row_step + row_off;
-    ti.n0 = (int)(r2 / gsz) * BN;
-    ti.row_end = cu.row_end;
-    ti.kg0 = (int)((int64_t)kc * cu.nk / cu.kch);
-    ti.kg1 = (int)((int64_t)(kc + 1) * cu.nk / cu.kch);
+    const int64_t col = div_small(r2, gsz);
+    TileInfo ti;
+    ti.t = cu.t_begin + (int)t;
+    ti.m0 = cu.row_begin + (first_m + (int)(r2 - col * gsz)) * row_step + row_off;
+    ti.n0 = (int)col * BN;
     return ti;
 }
 
@@ -816,13 +836,14 @@ __device__ __forceinline__ void add_private(float *__restrict__ mb, const uint32
 
 using LaunchArgs = TcLaunchArgs;
 
-// Sum of 16 per-lane values over the warp's 32 lanes by recursive halving: each exchange
-// sends the half of the values this lane does not keep; after four steps lanes 2m and
-// 2m + 1 hold partial sums of value m, which the last exchange adds.
-__device__ __forceinline__ float warp_sum16(float (&z)[16], int lane)
+// Sum of 8 per-lane values over the warp's 32 lanes by recursive halving: each exchange
+// sends the half of the values this lane does not keep; after three steps lanes
+// 4m .. 4m + 3 hold partial sums of value m (bits 4, 3, 2 of the lane, highest first), which
+// the last two exchanges add.
+__device__ __forceinline__ float warp_sum8(float (&z)[8], int lane)
 {
 #pragma unroll
-    for (int hh = 8, o = 16; hh >= 1; hh >>= 1, o >>= 1) {
+    for (int hh = 4, o = 16; hh >= 1; hh >>= 1, o >>= 1) {
         const bool up = (lane & o) != 0;
 #pragma unroll
         for (int k = 0; k < hh; ++k) {
@@ -831,7 +852,21 @@ __device__ __forceinline__ float warp_sum16(float (&z)[16], int lane)
             z[k] = keep + __shfl_xor_sync(0xffffffffu, send, o);
         }
     }
-    return z[0] + __shfl_xor_sync(0xffffffffu, z[0], 1);
+    const float w = z[0] + __shfl_xor_sync(0xffffffffu, z[0], 2);
+    return w + __shfl_xor_sync(0xffffffffu, w, 1);
+}
+
+__device__ __forceinline__ float warp_min(float x)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) x = fminf(x, __shfl_xor_sync(0xffffffffu, x, o));
+    return x;
+}
+__device__ __forceinline__ float warp_max(float x)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) x = fmaxf(x, __shfl_xor_sync(0xffffffffu, x, o));
+    return x;
 }
 
 // K block of a work item before which sub-pass g (of G) of the previous item's phase
@@ -859,16 +894,22 @@ __device__ __forceinline__ int phase_slot(int g, int nk, int G)
 // epilogue bins them.  Both CTAs walk the same fixed order of work items; the second
 // CTA's epilogue warps release accumulators and phase products on the first CTA's
 // barriers.
+__host__ __device__ constexpr bool phase_ok(int BN) { return 2 * BN + kPCols <= (int)kTmemAlloc; }
+__host__ __device__ constexpr int readout_warps(int BN) { return phase_ok(BN) ? 4 : 0; }
+__host__ __device__ constexpr int tc_threads(int BN, int EW)
+{
+    return 32 * (3 + EW + readout_warps(BN));
+}
+
 template <int FORM, int BN, int SWB, int EW, int CG>
-__global__ void __launch_bounds__(64 + 32 * EW, 1) pc_tc_kernel(const __grid_constant__ LaunchArgs args)
+__global__ void __launch_bounds__(tc_threads(BN, EW), 1) pc_tc_kernel(const __grid_constant__ LaunchArgs args)
 {
     constexpr int kEpiWarps = EW;
     constexpr int kEpiThreads = 32 * EW;
     constexpr int kBinStride = bin_stride(EW);
     constexpr int kHalves = EW / 4;
     constexpr int kChunks = BN / 32;                                 // 32-column chunks
-    constexpr int kColM = (BN + kEpiThreads - 1) / kEpiThreads;      // columns per thread
-    static_assert(kChunks <= 8, "chunk boxes of a tile (and one lane per chunk)");
+    static_assert(kChunks <= 8, "one lane per column chunk");
     constexpr bool kTF32 = FORM == ASD_TF32;
     constexpr int kPlanes = FORM == ASD_SPLIT_BF16 ? 2 : 1;
     constexpr uint32_t kABytes = kBM * SWB;
@@ -884,7 +925,8 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) pc_tc_kernel(const __grid_con
     // 128 x 128 x BN product P = G W with W[c][o] = cos / sin(q_o . r_c) of the tile's
     // columns, streamed through the operand ring (64 columns c per stage).  Split-BF16 and
     // TF32 issue hi*hi + hi*lo + lo*hi (the FP32-accurate sum); BF16 issues hi*hi.
-    constexpr bool kPhaseOK = 2 * BN + kPCols <= (int)kTmemAlloc;
+    constexpr bool kPhaseOK = phase_ok(BN);
+    constexpr int kRoWarps = readout_warps(BN);
     constexpr int kWPlanes = FORM == ASD_BF16 ? 1 : 2;
     constexpr int kWStages = BN / 64;          // W stages per pass (64 columns c each)
     constexpr uint32_t kWB = kWBytes / CG;     // one W plane of this CTA (its output half)
@@ -903,19 +945,21 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) pc_tc_kernel(const __grid_con
     const EpiLayout EL = epi_layout(args.VB, args.NB, args.NQ, BN, EW, args.det);
     uint64_t *bars = reinterpret_cast<uint64_t *>(epi + EL.total);
     // bars: full[stages], empty[stages], tfull[2], tempty[2], drain, wqfull[kWQ],
-    // wqempty[kWQ], conv, pfull, pempty, tmm[2]; then the work ring wq[kWQ] and the TMEM
-    // address slot
+    // wqempty[kWQ], conv, pfull, pempty, tmm[2], gfull[2], gempty[2]; then the work ring
+    // wq[kWQ] and the TMEM address slot
     const uint32_t wqfull0 = saddr(bars + 2 * stages + 5);
     const uint32_t wqempty0 = saddr(bars + 2 * stages + 5 + kWQ);
     // conv: the epilogue has stored a chunk's G as BF16 hi / lo (one arrival per warp);
-    // pfull: the phase product to be read out is complete; pempty: the epilogue has read
-    // it; tmm[a]: the phase product of the chunk in accumulator a is complete, so the
+    // pfull: the phase product to be read out is complete; pempty: the read-out warps have
+    // read it; tmm[a]: the phase product of the chunk in accumulator a is complete, so the
     // buffer is free (for phase work the MMA thread releases the accumulator, not the
-    // epilogue)
+    // epilogue); gfull / gempty: a tile's geometry buffer is filled / has been used
     const uint32_t conv = saddr(bars + 2 * stages + 5 + 2 * kWQ);
     const uint32_t pfull = conv + 8, pempty = conv + 16, tmm0 = conv + 24;
-    volatile int64_t *wq = reinterpret_cast<volatile int64_t *>(bars + 2 * stages + 10 + 2 * kWQ);
-    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + 2 * stages + 10 + 3 * kWQ);
+    const uint32_t gfull0 = conv + 40, gempty0 = conv + 56;
+    volatile WorkSlot *wq = reinterpret_cast<volatile WorkSlot *>(
+        (reinterpret_cast<uintptr_t>(bars + 2 * stages + 14 + 2 * kWQ) + 15) & ~(uintptr_t)15);
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(const_cast<WorkSlot *>(wq + kWQ));
     const uint32_t full0 = saddr(bars), empty0 = saddr(bars + stages);
     const uint32_t tfull0 = saddr(bars + 2 * stages), tempty0 = saddr(bars + 2 * stages + 2);
     const uint32_t drain = saddr(bars + 2 * stages + 4);
@@ -941,16 +985,32 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) pc_tc_kernel(const __grid_con
         mbar_init(drain, 1);
         for (int k = 0; k < kWQ; ++k) {
             mbar_init(wqfull0 + 8 * k, 1);
-            // released by the MMA thread (the first CTA of a pair only) and one lane of
-            // every epilogue warp
-            mbar_init(wqempty0 + 8 * k, (leader ? 1 : 0) + kEpiWarps);
+            // released by the MMA thread (the first CTA of a pair only), one lane of every
+            // epilogue and read-out warp and the geometry warp
+            mbar_init(wqempty0 + 8 * k, (leader ? 1 : 0) + kEpiWarps + 1 + kRoWarps);
         }
         mbar_init(conv, kEpiWarps * CG);
         mbar_init(pfull, 1);
-        mbar_init(pempty, kEpiWarps * CG);
+        mbar_init(pempty, 4 * CG);
         mbar_init(tmm0, 1);
         mbar_init(tmm0 + 8, 1);
+        for (int a = 0; a < 2; ++a) {
+            mbar_init(gfull0 + 8 * a, 1);
+            mbar_init(gempty0 + 8 * a, kEpiWarps);
+        }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    // descriptors of the first problem (a batch's other problems fetch theirs when they come)
+    if (warp == 0) {
+        const CUtensorMap *maps = &args.probs->mapA[0][0];
+        constexpr int kMaps = 2 * kMaxCopies + 4;   // mapA, mapB, mapW
+        const int n_copies = args.one.n_copies;
+        if (lane < kMaps && (lane >= 2 * kMaxCopies || lane % kMaxCopies < n_copies) &&
+            (lane < 2 * kMaxCopies + 2 || args.one.npass > 0) &&
+            !(kPlanes == 1 && ((lane >= kMaxCopies && lane < 2 * kMaxCopies) ||
+                               lane == 2 * kMaxCopies + 1)))
+            asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(maps + lane))
+                         : "memory");
     }
     if (warp == 1) tmem_alloc<CG>(saddr(tmem_slot), kTmemAlloc);
     tc_before();
@@ -1014,41 +1074,74 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) pc_tc_kernel(const __grid_con
             // k n + (c + k) mod n.  Without the rotation a raster group of a multiple of n
             // items would put every CTA on the same columns in every group, so the costly
             // column tiles would always land on the same CTAs.
-            int64_t tau = 0;
-            int kci = 0, kch = 0;
+            auto claim = [&]() -> int64_t {
+                if (args.counter && CG == 1)
+                    return n_ctas + (int64_t)atomicAdd(args.counter, 1ull);
+                const int64_t r = n_claimed * n_ctas + (cid + n_claimed) % n_ctas;
+                ++n_claimed;
+                return r;
+            };
+            // (the first items are the CTAs' numbers: no claim to wait for)
+            int64_t tau_next = args.counter && CG == 1 ? cid : claim();
+            // the next item, once decoded (p = -1: none left), and the current one
+            int p_next = -2, p_cur = -1, kci = 0, kch = 0;
+            TileInfo t_next = {}, ti = {};
+            auto take = [&]() {
+                const int64_t tau = tau_next;
+                if (tau >= args.total_tiles) {
+                    p_next = -1;
+                    return;
+                }
+                tau_next = claim();   // its reply is not waited for until the next call
+                t_next = decode(cu, probs, args.n_probs, args.one, args.ov, tau, BN, row_step,
+                                row_off);
+                p_next = cu.p;
+            };
+            take();
+            WorkCursor wc;   // the current item's problem (cu may be one item ahead)
             for (int64_t v = 0; ok; ++v) {
                 const int qs = (int)(v % kWQ);
                 // the next chunk of the current item, or the first of a new one
                 if (++kci >= kch) {
-                    tau = args.counter && CG == 1
-                              ? (int64_t)atomicAdd(args.counter, 1ull)
-                              : n_claimed * n_ctas + (cid + n_claimed) % n_ctas;
-                    ++n_claimed;
-                    if (tau >= args.total_tiles) tau = -1;
+                    if (p_next == -2) take();
+                    if (p_next >= 0 && p_next != p_cur) wc = cu;
+                    p_cur = p_next;
+                    ti = t_next;
+                    p_next = -2;
                     kci = 0;
-                    kch = tau < 0 ? 1
-                                  : probs[decode(cu, probs, args.n_probs, args.ov, tau, 0, BN,
-                                                 row_step, row_off).p].k_chunks;
+                    kch = p_cur < 0 ? 1 : wc.kch;
                 }
-                // publish the sub-item (tau 256 + chunk; -1: none left) once its ring slot
-                // is free
+                const int kg0 = p_cur < 0 ? 0 : (int)div_small((int64_t)kci * wc.nk, kch);
+                const int kg1 = p_cur < 0 ? 0 : (int)div_small((int64_t)(kci + 1) * wc.nk, kch);
+                // publish the sub-item once its ring slot is free
                 if (!mbar_wait(wqempty0 + 8 * qs, (uint32_t)((v / kWQ) & 1) ^ 1u, args.err,
                                DEV_TIMEOUT_TMA)) {
                     ok = false;
                     break;
                 }
-                wq[qs] = tau < 0 ? -1 : tau * 256 + kci;
+                volatile WorkSlot &w = wq[qs];
+                w.p = p_cur;
+                w.t = ti.t;
+                w.m0 = ti.m0;
+                w.n0 = ti.n0;
+                w.row_end = wc.row_end;
+                w.kci = kci;
+                w.last = kci == kch - 1;
+                w.nk = kg1 - kg0;
                 mbar_arrive(wqfull0 + 8 * qs);  // release: the slot is visible to the waiters
-                if (tau < 0) break;
-                const TileInfo ti =
-                    decode(cu, probs, args.n_probs, args.ov, tau, kci, BN, row_step, row_off);
-                const TcProblem &P = probs[ti.p];
-                const int nk = ti.kg1 - ti.kg0;
+                if (p_cur < 0) break;
+                const TcProblem &P = probs[p_cur];
+                const int nk = kg1 - kg0;
+                // decode the next item in the middle of this one's last chunk
+                const int kg_take = kci == kch - 1 ? kg0 + nk / 2 : -1;
+                // sample and K block inside it, and the operand window of that sample
+                int s = kg0 / wc.nkb, kb = kg0 - s * wc.nkb;
+                int xw = s * wc.F3 + 3 * ti.t, c = xw % wc.n_copies;
                 int g = 0;
-                for (int kg = ti.kg0; kg < ti.kg1 && ok; ++kg) {
+                for (int kg = kg0; kg < kg1 && ok; ++kg) {
                     if constexpr (kPhaseOK) {
                         while (pend_p >= 0 && g < pend_G &&
-                               kg - ti.kg0 == phase_slot(g, nk, pend_G)) {
+                               kg - kg0 == phase_slot(g, nk, pend_G)) {
                             if (!load_sub(g++)) {
                                 ok = false;
                                 break;
@@ -1056,10 +1149,6 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) pc_tc_kernel(const __grid_con
                         }
                         if (!ok) break;
                     }
-                    const int s = kg / P.nkb, kb = kg % P.nkb;
-                    const int xw = s * P.F3 + 3 * ti.t;
-                    const int c = xw % P.n_copies;
-
                     if (!mbar_wait(empty0 + 8 * stage, phase ^ 1, args.err, DEV_TIMEOUT_TMA)) {
                         ok = false;
                         break;
@@ -1075,22 +1164,29 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) pc_tc_kernel(const __grid_con
                             tma_load_2d_pair(saddr(st + pl * kABytes), &P.mapA[pl][c],
                                              lead(fb), xw - c + kb * kBK, ti.m0);
                             tma_load_2d_pair(saddr(st + kPlanes * kABytes + pl * kBBytes),
-                                             &P.mapB[pl], lead(fb), s * P.Kseg + kb * kBK,
+                                             &P.mapB[pl], lead(fb), s * wc.Kseg + kb * kBK,
                                              nb0);
                         } else {
                             tma_load_2d(saddr(st + pl * kABytes), &P.mapA[pl][c], fb,
                                         xw - c + kb * kBK, ti.m0);
                             tma_load_2d(saddr(st + kPlanes * kABytes + pl * kBBytes),
-                                        &P.mapB[pl], fb, s * P.Kseg + kb * kBK, nb0);
+                                        &P.mapB[pl], fb, s * wc.Kseg + kb * kBK, nb0);
                         }
                     }
                     next_stage();
+                    if (++kb == wc.nkb) {
+                        kb = 0;
+                        ++s;
+                        xw += wc.F3;
+                        c = xw % wc.n_copies;
+                    }
+                    if (kg == kg_take) take();
                 }
                 pend_p = -1;
-                if (kPhaseOK && P.epi.n_q > 0) {
-                    pend_p = ti.p;
+                if (kPhaseOK && wc.npass > 0) {
+                    pend_p = p_cur;
                     pend_n0 = ti.n0;
-                    pend_G = P.epi.npass * kWStages;
+                    pend_G = wc.npass * kWStages;
                 }
             }
             // the last item's phase sub-passes
@@ -1125,7 +1221,7 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) pc_tc_kernel(const __grid_con
             uint32_t phase = 0;
             uint32_t v = 0;
             bool ok = true;
-            WorkCursor cu;
+            int p_cur = -1, npass = 0;
             // previous sub-item with phase sub-passes still to issue: its accumulator
             // buffer and sub-pass count; whether its product adds to P (a later K chunk of
             // a tile with one pass: P sums the chunks and is read out once) and whether it
@@ -1194,14 +1290,14 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) pc_tc_kernel(const __grid_con
                     ok = false;
                     break;
                 }
-                const int64_t tau = wq[qs];
+                const int p = wq[qs].p, kci = wq[qs].kci, last = wq[qs].last, nk = wq[qs].nk;
                 mbar_arrive(wqempty0 + 8 * qs);
-                if (tau < 0) break;
-                const int kci = (int)(tau & 255);
-                const TileInfo ti = decode(cu, probs, args.n_probs, args.ov, tau >> 8, kci, BN,
-                                           row_step, row_off);
-                const TcProblem &P = probs[ti.p];
-                const bool phs = kPhaseOK && P.epi.n_q > 0;
+                if (p < 0) break;
+                if (p != p_cur) {
+                    p_cur = p;
+                    npass = args.n_probs == 1 ? args.one.npass : probs[p].dims.npass;
+                }
+                const bool phs = kPhaseOK && npass > 0;
                 const uint32_t acc = v & 1;
                 // wait until the accumulator's previous chunk has released it
                 if (rel[acc] == 1 && !mbar_wait(tempty0 + 8 * acc, n_te[acc]++ & 1, args.err,
@@ -1217,10 +1313,8 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) pc_tc_kernel(const __grid_con
                 rel[acc] = phs ? 2 : 1;
                 tc_after();
                 const uint32_t d = tmem + acc * BN;
-                const int nk = ti.kg1 - ti.kg0;
                 int g = 0;
-                for (int kg = ti.kg0; kg < ti.kg1; ++kg) {
-                    const int kb = kg - ti.kg0;  // 0 for the first block of this chunk
+                for (int kb = 0; kb < nk; ++kb) {  // 0: the first block of this chunk
                     if constexpr (kPhaseOK) {
                         while (pend_acc >= 0 && g < pend_G && kb == phase_slot(g, nk, pend_G)) {
                             if (!issue_sub(g++)) {
@@ -1263,11 +1357,11 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) pc_tc_kernel(const __grid_con
                 pend_acc = -1;
                 if (phs) {
                     // one pass: P sums the tile's chunks and is read out after the last
-                    const bool across = P.epi.npass == 1;
+                    const bool across = npass == 1;
                     pend_acc = (int)acc;
-                    pend_G = P.epi.npass * kWStages;
+                    pend_G = npass * kWStages;
                     pend_add = across && kci > 0;
-                    pend_done = !across || kci == P.k_chunks - 1;
+                    pend_done = !across || last;
                 }
             }
             // the last item's phase sub-passes
@@ -1277,6 +1371,329 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) pc_tc_kernel(const __grid_con
             tc_commit<CG>(drain);
             mbar_wait(drain, 0, args.err, DEV_TIMEOUT_MMA);
         }
+    } else if (warp == 2 + kEpiWarps) {
+        // ======================= geometry =======================
+        // (on the epilogue warps, behind two barriers and several dependent global loads,
+        // this took 5 to 10 thousand cycles of each tile; the epilogue now waits for it less
+        // than 1 thousand)
+        uint32_t item = 0;  // tiles prepared
+        for (uint32_t v = 0;; ++v) {
+            const int qs = (int)(v % kWQ);
+            bool ok = mbar_wait(wqfull0 + 8 * qs, (v / kWQ) & 1, args.err, DEV_TIMEOUT_EPI);
+            if (!__all_sync(0xffffffffu, ok)) break;
+            const int p = wq[qs].p, m0 = wq[qs].m0, n0 = wq[qs].n0, row_end = wq[qs].row_end;
+            const bool first = wq[qs].kci == 0;
+            __syncwarp();
+            if (lane == 0) mbar_arrive(wqempty0 + 8 * qs);
+            if (p < 0) break;
+            if (!first) continue;
+            const uint32_t gb = item & 1;
+            ok = mbar_wait(gempty0 + 8 * gb, ((item >> 1) & 1) ^ 1u, args.err, DEV_TIMEOUT_EPI);
+            if (!__all_sync(0xffffffffu, ok)) break;
+            ++item;
+            const EpiParams &E = probs[p].epi;
+            const int N = probs[p].dims.N;
+            float *cg = reinterpret_cast<float *>(epi + EL.geo) + gb * 3 * BN;
+            const bool lattice = E.geom == ASD_GEOM_LATTICE;
+            // columns (past the last site: its geometry, with zero products), one per lane
+            // and 32-column chunk
+            float cx[kChunks][3];
+#pragma unroll
+            for (int m = 0; m < kChunks; ++m) {
+                const int c = 32 * m + lane, j = min(n0 + c, N - 1);
+                if (lattice) {
+                    const int4 g = E.coords[j];
+                    if (E.fast && (E.NW + 1) * kBinStride <= 65536) {
+                        reinterpret_cast<uint32_t *>(cg)[c] =
+                            (uint32_t)g.x | ((uint32_t)g.y << 8) | ((uint32_t)g.z << 16);
+                    } else {
+                        cg[c] = __int_as_float(g.x);
+                        cg[BN + c] = __int_as_float(g.y);
+                        cg[2 * BN + c] = __int_as_float(g.z);
+                    }
+                    cx[m][0] = (float)g.x;
+                    cx[m][1] = (float)g.y;
+                    cx[m][2] = (float)g.z;
+                } else {
+                    const float4 g = E.pos[j];
+                    cg[c] = cx[m][0] = g.x;
+                    cg[BN + c] = cx[m][1] = g.y;
+                    cg[2 * BN + c] = cx[m][2] = g.z;
+                }
+            }
+            TileWindow tw = {0, 0, E.NW, E.n_bins, kChunks, E.n_bins - 1,
+                             !E.use_window && E.pos_ok, 0};
+            if (E.use_window) {
+                // boxes of the rows inside the range and of each column chunk
+                float rl[3] = {3e38f, 3e38f, 3e38f}, rh[3] = {-3e38f, -3e38f, -3e38f};
+                for (int m = 0; m < kBM / 32; ++m) {
+                    const int i = m0 + 32 * m + lane;
+                    if (i < row_end) {
+                        float r[3];
+                        if (lattice) {
+                            const int4 g = E.coords[i];
+                            r[0] = (float)g.x;
+                            r[1] = (float)g.y;
+                            r[2] = (float)g.z;
+                        } else {
+                            const float4 g = E.pos[i];
+                            r[0] = g.x;
+                            r[1] = g.y;
+                            r[2] = g.z;
+                        }
+#pragma unroll
+                        for (int a = 0; a < 3; ++a) {
+                            rl[a] = fminf(rl[a], r[a]);
+                            rh[a] = fmaxf(rh[a], r[a]);
+                        }
+                    }
+                }
+                // (lane m keeps the box of chunk m)
+                float bl[3], bh[3], cl[3], ch[3];
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {
+                    rl[a] = warp_min(rl[a]);
+                    rh[a] = warp_max(rh[a]);
+                    bl[a] = cl[a] = 3e38f;
+                    bh[a] = ch[a] = -3e38f;
+#pragma unroll
+                    for (int m = 0; m < kChunks; ++m) {
+                        const float lo = warp_min(cx[m][a]), hi = warp_max(cx[m][a]);
+                        if (lane == m) {
+                            bl[a] = lo;
+                            bh[a] = hi;
+                        }
+                        cl[a] = fminf(cl[a], lo);
+                        ch[a] = fmaxf(ch[a], hi);
+                    }
+                }
+                auto box_d2 = [&](const float (&lo)[3], const float (&hi)[3], float &dmin,
+                                  float &dmax) {
+                    dmin = dmax = 0.f;
+#pragma unroll
+                    for (int a = 0; a < 3; ++a) {
+                        float gap = fmaxf(0.f, fmaxf(lo[a] - rh[a], rl[a] - hi[a]));
+                        if (lattice && E.periodic) {
+                            const float L = a == 0 ? E.Lx : a == 1 ? E.Ly : E.Lz;
+                            gap = fminf(gap, fmaxf(0.f, fmaxf(lo[a] + L - rh[a], rl[a] - (hi[a] + L))));
+                            gap = fminf(gap, fmaxf(0.f, fmaxf(lo[a] - L - rh[a], rl[a] - (hi[a] - L))));
+                        }
+                        const float far = fmaxf(hi[a] - rl[a], rh[a] - lo[a]);
+                        dmin += gap * gap;
+                        dmax += far * far;
+                    }
+                };
+                auto lo_bin = [&](float d2) {
+                    return max(0, bin_of_d2(d2 * 0.999f, E.inv_w, E.n_bins, E.thr) - 1);
+                };
+                auto hi_bin = [&](float d2) {
+                    return min(E.n_bins - 1,
+                               bin_of_d2(d2 * 1.001f + 1e-30f, E.inv_w, E.n_bins, E.thr) + 1);
+                };
+                float dmin, dmax;
+                box_d2(cl, ch, dmin, dmax);
+                tw.blo = lo_bin(dmin);
+                if (!lattice) {
+                    tw.bhi = hi_bin(dmax);
+                    tw.nwp = tw.bhi - tw.blo + 1;
+                    tw.fit = E.pos_ok && tw.nwp <= E.NW;
+                    if (!tw.fit && E.pos_ok) {
+                        // bins of each 32-column chunk (lane c computes chunk c), then the
+                        // first split of the chunks into two windows that together fit
+                        box_d2(bl, bh, dmin, dmax);
+                        const int lo_c = lane < kChunks ? lo_bin(dmin) : 0;
+                        const int hi_c = lane < kChunks ? hi_bin(dmax) : 0;
+                        int lo[kChunks], hi[kChunks];
+#pragma unroll
+                        for (int c = 0; c < kChunks; ++c) {
+                            lo[c] = __shfl_sync(0xffffffffu, lo_c, c);
+                            hi[c] = __shfl_sync(0xffffffffu, hi_c, c);
+                        }
+                        // one window over the chunks' bins (narrower than the tile's
+                        // box); only when that does not fit, two windows, which are then
+                        // disjoint (two overlapping ones would span no more than their
+                        // sum), so no bin has two private rows
+                        int l0 = 1 << 30, h0 = -1;
+#pragma unroll
+                        for (int c = 0; c < kChunks; ++c) {
+                            l0 = min(l0, lo[c]);
+                            h0 = max(h0, hi[c]);
+                        }
+                        int best = E.NW + 1, b1 = 0, b2 = 0, bn = 0, bs = kChunks;
+                        if (h0 - l0 + 1 <= E.NW) {
+                            best = h0 - l0 + 1;
+                            b1 = l0;
+                            bn = E.NW;
+                        }
+#pragma unroll
+                        for (int sp = 1; sp < kChunks && best > E.NW; ++sp) {
+                            int l1 = 1 << 30, h1 = -1, l2 = 1 << 30, h2 = -1;
+#pragma unroll
+                            for (int c = 0; c < kChunks; ++c) {
+                                if (c < sp) { l1 = min(l1, lo[c]); h1 = max(h1, hi[c]); }
+                                else { l2 = min(l2, lo[c]); h2 = max(h2, hi[c]); }
+                            }
+                            const int need = (h1 - l1 + 1) + (h2 - l2 + 1);
+                            if (need < best) {
+                                best = need;
+                                b1 = l1;
+                                bn = h1 - l1 + 1;
+                                b2 = l2;
+                                bs = sp;
+                            }
+                        }
+                        if (best <= E.NW) {
+                            tw.fit = 1;
+                            tw.nwp = best;
+                            tw.blo = b1;
+                            tw.blo2 = b2;
+                            tw.n1 = bn;
+                            tw.split = bs;
+                        }
+                    }
+                }
+            }
+            if (lane == 0) reinterpret_cast<TileWindow *>(epi + EL.win)[gb] = tw;
+            __syncwarp();   // (every lane's stores before the arrive's release)
+            if (lane == 0) mbar_arrive(gfull0 + 8 * gb);
+        }
+    } else if (kPhaseOK && warp > 2 + kEpiWarps) {
+        // ======================= phase read-out =======================
+        // Phase product of each pass: P[r][o] = sum_c G_rc W_co, u = P[.][0:64) (cosine column
+        // weights), v = P[.][64:128) (sine).  Row r adds cos(q.r_i) u + sin(q.r_i) v (cosine
+        // part) and sin(q.r_i) u - cos(q.r_i) v (sine part), the angle-difference identities
+        // of Eq. 6's weight; a warp sums its 32 rows by recursive halving and adds them to
+        // its FP64 sums.  Warps of their own: the 64 row weights of a row come from L2 behind
+        // the operand streams, and the read-out on the epilogue warps, between the binning
+        // of two tiles, took 8 to 12 thousand cycles of each tile (48^3 glass BF16, the
+        // epilogue's other parts as now: 122 -> 100 ms, 32^3 glass split-BF16 21.3 -> 19.3); here the weights of the next read-out load
+        // while its product is still to come, and the binning does not wait.  One pass:
+        // P sums the tile's K chunks and is read out after the last; several passes: each is
+        // read out per chunk.
+        const int q4 = warp & 3;   // TMEM lane quarter of this warp
+        double *qa = reinterpret_cast<double *>(epi + EL.qacc) + q4 * args.NQ;
+        long long *qai = reinterpret_cast<long long *>(qa);   // deterministic mode
+        for (int k = lane; k < args.NQ; k += 32) qa[k] = 0.0;
+        __syncwarp();
+        const uint32_t pt = tmem + ((uint32_t)(q4 * 32) << 16) + 2 * BN;
+        int cur_p = -1, cur_t = -1, N = 0, n_q = 0, npass = 0, parts = 1, n_t = 0;
+        int64_t ld = 0;
+        const float2 *csT = nullptr;
+        double fscale = 0.0, *Qs = nullptr;
+        long long *Qf = nullptr;
+        bool det = false;
+        uint32_t n_pass = 0;   // passes read out (parity of pfull)
+        // the sums of the current (problem, t), added to the outputs when it changes
+        auto flush_q = [&]() {
+            if (cur_p < 0 || n_q == 0) return;
+            const bool t_ok = ASD_INB((unsigned)cur_t < (unsigned)n_t, BND_WORK, args.err);
+            for (int k = lane; k < n_q * parts; k += 32) {
+                const int64_t o = (int64_t)cur_t * n_q * parts + k;
+                if (det) {
+                    if (qai[k] != 0 && t_ok) add_fixed(&Qf[o], qai[k]);
+                } else if (qa[k] != 0.0 && t_ok) {
+                    atomicAdd(&Qs[o], qa[k]);
+                }
+                qa[k] = 0.0;
+            }
+            __syncwarp();
+        };
+        bool ok = true;
+        for (uint32_t v = 0; ok; ++v) {
+            const int qs = (int)(v % kWQ);
+            ok = __all_sync(0xffffffffu, mbar_wait(wqfull0 + 8 * qs, (v / kWQ) & 1, args.err,
+                                                   DEV_TIMEOUT_EPI));
+            if (!ok) break;
+            const int p = wq[qs].p, t = wq[qs].t, i = wq[qs].m0 + q4 * 32 + lane;
+            const bool row_ok = i < wq[qs].row_end, last = wq[qs].last != 0;
+            __syncwarp();
+            if (lane == 0) mbar_arrive(wqempty0 + 8 * qs);
+            if (p < 0) break;
+            if (p != cur_p || t != cur_t) flush_q();
+            if (p != cur_p) {
+                const EpiParams &E = probs[p].epi;
+                N = probs[p].dims.N;
+                n_t = probs[p].dims.n_t;
+                n_q = E.n_q;
+                npass = E.npass;
+                parts = E.q_parts;
+                csT = E.csT;
+                ld = E.cs_ld;
+                det = E.fix_scale != nullptr;
+                fscale = det ? *E.fix_scale : 0.0;
+                Qs = args.ov.active ? args.ov.Sq_sum : E.Sq_sum;
+                Qf = E.Sq_fix;
+            }
+            cur_p = p;
+            cur_t = t;
+            if (n_q == 0 || (npass == 1 && !last)) continue;
+            // (rows past the range hold zeros in P)
+            const float2 *cs = csT + (row_ok ? i : N - 1);
+            for (int q0 = 0; ok && q0 < npass * kPhaseQ; q0 += 32) {
+                // 32 q-vectors (half a pass) at a time; the table has a row per q, so a
+                // warp's 32 consecutive sites read two or three lines per q.  Rows past n_q
+                // up to the padding are zero.
+                float2 cw[32];
+#pragma unroll
+                for (int k = 0; k < 32; ++k)
+                    if (q0 + (k & 16) < n_q) cw[k] = cs[(int64_t)(q0 + k) * ld];
+                    else cw[k] = make_float2(0.f, 0.f);
+                const int h = q0 & 32;   // second half of the pass
+                if (h == 0) {
+                    ok = __all_sync(0xffffffffu,
+                                    mbar_wait(pfull, n_pass & 1, args.err, DEV_TIMEOUT_EPI));
+                    if (!ok) break;
+                    ++n_pass;
+                    tc_after();
+                }
+                float xs = 0.f, ys = 0.f;   // this lane's q of the 32
+#pragma unroll
+                for (int j = 0; j < 32; j += 8) {
+                    uint32_t u[8], w[8];
+                    tmem_ld8(pt + h + j, u);
+                    tmem_ld8(pt + kPhaseQ + h + j, w);
+                    tmem_wait8x2(u, w);
+                    float x[8];
+#pragma unroll
+                    for (int k = 0; k < 8; ++k)
+                        x[k] = fmaf(cw[j + k].x, __uint_as_float(u[k]),
+                                    cw[j + k].y * __uint_as_float(w[k]));
+                    const float xj = warp_sum8(x, lane);
+                    // (every fourth lane group holds one of the eight; lane & 3 picks j, so
+                    // one FP64 conversion and add serves all 32)
+                    if ((lane & 3) == (j >> 3)) xs = xj;
+                    if (parts == 2) {
+#pragma unroll
+                        for (int k = 0; k < 8; ++k)
+                            x[k] = fmaf(cw[j + k].y, __uint_as_float(u[k]),
+                                        -cw[j + k].x * __uint_as_float(w[k]));
+                        const float yj = warp_sum8(x, lane);
+                        if ((lane & 3) == (j >> 3)) ys = yj;
+                    }
+                }
+                const int qme = q0 + (lane & 3) * 8 + ((lane >> 4) & 1) * 4 +
+                                ((lane >> 3) & 1) * 2 + ((lane >> 2) & 1);
+                if (qme < n_q && ASD_INB((qme + 1) * parts <= args.NQ, BND_Q, args.err)) {
+                    if (det) qai[qme * parts] += to_fixed((double)xs, fscale);
+                    else qa[qme * parts] += (double)xs;
+                    if (parts == 2) {
+                        if (det) qai[qme * 2 + 1] += to_fixed((double)ys, fscale);
+                        else qa[qme * 2 + 1] += (double)ys;
+                    }
+                }
+                // P read: the next pass (or item) may overwrite it
+                if (h == 32) {
+                    tc_before();
+                    __syncwarp();
+                    if (lane == 0) {
+                        if constexpr (CG == 2) mbar_arrive_cl(lead(pempty));
+                        else mbar_arrive(pempty);
+                    }
+                }
+            }
+        }
+        __syncwarp();
+        if (ok) flush_q();
     } else {
         // ======================= epilogue =======================
         const int et = threadIdx.x - 64;          // 0..127
@@ -1289,32 +1706,24 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) pc_tc_kernel(const __grid_con
         float *bins = reinterpret_cast<float *>(epi + EL.var);
         float *fb = reinterpret_cast<float *>(epi + EL.fb);
         double *cacc = reinterpret_cast<double *>(epi + EL.cacc);
-        double *qacc = reinterpret_cast<double *>(epi + EL.qacc);
         // the same arrays as 64-bit fixed point (problems in the deterministic mode)
         long long *fbi = reinterpret_cast<long long *>(epi + EL.fb);
         long long *cacci = reinterpret_cast<long long *>(epi + EL.cacc);
-        long long *qacci = reinterpret_cast<long long *>(epi + EL.qacc);
-        float *colgeo = reinterpret_cast<float *>(epi + EL.colgeo);
-        uint32_t *colpk = reinterpret_cast<uint32_t *>(epi + EL.colpk);
-        float *boxred = reinterpret_cast<float *>(epi + EL.boxred);
-        float *chbox = boxred + kEpiWarps * 12;
+        // the current problem's parameters and fixed-point scale (0: FP sums)
+        const EpiParams &E = *reinterpret_cast<const EpiParams *>(epi + EL.par);
+        double fscale = 0.0;
+        bool det = false;
         float *thr_s = bins;
         for (int k = et; k < args.NB; k += kEpiThreads) {
             if (args.det) fbi[k] = 0;
             else fb[k] = 0.f;
             cacc[k] = 0.0;  // (all-zero bits: also fixed-point zero)
         }
-        for (int k = et; k < 2 * args.NQ; k += kEpiThreads) qacc[k] = 0.0;
 
-        int cur_p = -1, cur_t = -1, tab_p = -1;
-        WorkCursor cu;
+        int cur_p = -1, cur_t = -1, N = 0;
         // fast lattice binning also needs the private-bin offsets of this launch (the
         // largest window of a batch, plus its trash row) to fit the 16-bit table entries
-        auto fast_ok = [&](const EpiParams &E) {
-            return E.fast && (E.NW + 1) * kBinStride <= 65536;
-        };
-        // phase passes read out so far (parity of pfull)
-        uint32_t n_pass = 0;
+        auto fast_ok = [&]() { return E.fast && (E.NW + 1) * kBinStride <= 65536; };
         // Store a 32-column chunk of this thread's accumulator row back as BF16 hi / lo
         // (16 columns each, two values per column, the even column in the low half):
         // the A operand of the phase product.  Rows past the range store zeros.
@@ -1335,24 +1744,20 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) pc_tc_kernel(const __grid_con
         };
         uint32_t v = 0;
         bool ok = true;
-        // geometry of the current tile, set by its first K chunk: this thread's row site,
-        // the bin window start and, for positions, whether the tile's bins fit the window
+        // the current tile: this thread's row site and its geometry, whether the row is in the
+        // range, the tile's columns and bin window(s)
         int4 ri = make_int4(0, 0, 0, 0);
         float4 rp = make_float4(0.f, 0.f, 0.f, 0.f);
-        int blo = 0, bhi_tile = 0;
-        bool pos_fit = false;
-        // positions: a tile whose columns span two far-apart groups of sites may take two
-        // windows, private rows [0, n1) for bins blo + k (column chunks before `split`) and
-        // rows [n1, nwp) for bins blo2 + k - n1 (the chunks from `split` on)
-        int blo2 = 0, n1 = 0, split = 0, nwp = 0;
+        int ic = 0;
+        bool row_ok = false;
+        uint32_t item = 0;   // tiles begun
+        const float *colgeo = nullptr;
+        TileWindow tw = {};
         // per-CTA FP64 sums of the current (problem, t), added to the outputs when it changes
         // (deterministic mode: fixed-point sums into the problem's fixed-point arrays)
         auto flush_acc = [&](int p, int t) {
-            const EpiParams &E = probs[p].epi;
             double *Cs = args.ov.active ? args.ov.C_sum : E.C_sum;
-            double *Qs = args.ov.active ? args.ov.Sq_sum : E.Sq_sum;
-            const bool det = E.fix_scale != nullptr;
-            const bool t_ok = ASD_INB((unsigned)t < (unsigned)probs[p].n_t, BND_WORK, args.err);
+            const bool t_ok = ASD_INB((unsigned)t < (unsigned)probs[p].dims.n_t, BND_WORK, args.err);
             for (int b = et; b < E.n_bins; b += kEpiThreads) {
                 const int64_t o = (int64_t)t * E.n_bins + b;
                 if (det) {
@@ -1362,293 +1767,118 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) pc_tc_kernel(const __grid_con
                 }
                 cacc[b] = 0.0;
             }
-            for (int q = et; q < E.n_q; q += kEpiThreads)
-                for (int part = 0; part < E.q_parts; ++part) {
-                    const int64_t o = ((int64_t)t * E.n_q + q) * E.q_parts + part;
-                    if (det) {
-                        if (qacci[2 * q + part] != 0 && t_ok)
-                            add_fixed(&E.Sq_fix[o], qacci[2 * q + part]);
-                    } else if (qacc[2 * q + part] != 0.0 && t_ok) {
-                        atomicAdd(&Qs[o], qacc[2 * q + part]);
-                    }
-                    qacc[2 * q + part] = 0.0;
-                }
+        };
+        bool bins_on = false;
+        // row geometry of the current tile (the load is in flight while the waits run)
+        auto load_row = [&]() {
+            // rows past the range (ragged tiles) read the geometry of a valid site and
+            // contribute zeros
+            if (E.geom == ASD_GEOM_LATTICE) ri = E.coords[ic];
+            else rp = E.pos[ic];
         };
         for (;; ++v) {
             const int qs = (int)(v % kWQ);
-            {
-                const bool gotq = mbar_wait(wqfull0 + 8 * qs, (v / kWQ) & 1, args.err,
-                                            DEV_TIMEOUT_EPI);
-                ok = epi_sync_and(gotq, kEpiThreads);
-                if (!ok) break;
+            const uint32_t acc = v & 1, use = v >> 1;
+            // the sub-item, its tile's geometry and its accumulator; every thread waits by
+            // itself, then all agree (a wait that gave up in one stops all)
+            bool got = mbar_wait(wqfull0 + 8 * qs, (v / kWQ) & 1, args.err, DEV_TIMEOUT_EPI);
+            int p = -1, t = 0, kci = 0, lst = 0;
+            bool new_t = false;
+            if (got) {
+                p = wq[qs].p;
+                t = wq[qs].t;
+                kci = wq[qs].kci;
+                lst = wq[qs].last;
+                if (kci == 0 && p >= 0) {
+                    const int i = wq[qs].m0 + r;
+                    row_ok = i < wq[qs].row_end;
+                    if (p == cur_p) {
+                        ic = row_ok ? i : N - 1;
+                        load_row();
+                    } else {
+                        ic = i;   // (N is read at the problem switch below)
+                    }
+                }
             }
-            const int64_t tau = wq[qs];
             __syncwarp();
-            if (lane == 0) mbar_arrive(wqempty0 + 8 * qs);
-            if (tau < 0) break;
-            const int kci = (int)(tau & 255);
-            const TileInfo ti = decode(cu, probs, args.n_probs, args.ov, tau >> 8, kci, BN,
-                                       row_step, row_off);
-            const TcProblem &P = probs[ti.p];
-            const EpiParams &E = P.epi;
-            // the first K chunk of a tile sets up its geometry and bin window; the chunks
-            // add into the same private bins, which the last one reduces
-            const bool first = kci == 0, last = kci == P.k_chunks - 1;
-            const int i = ti.m0 + r;
-            const bool row_ok = i < ti.row_end;
-            // rows past the range (ragged tiles) read the
-            // geometry of a valid site and contribute zeros
-            const int ic = row_ok ? i : P.N - 1;
-            const bool lattice = E.geom == ASD_GEOM_LATTICE;
-            // (a checked build also tests that the problem's bins and table fit the
-            // launch's per-problem region; if not, the problem is not binned)
-            const bool bins_on =
-                E.n_bins > 0 &&
-                ASD_INB(var_bytes(E.NW, E.n_bins, E.n_lut, EW) <= args.VB, BND_REGION, args.err);
-            // fixed-point scale of a problem in the deterministic mode (0: FP sums)
-            const double fscale = E.fix_scale ? *E.fix_scale : 0.0;
-            if (first) {
-                // bin thresholds of this problem, then the column geometry of this tile
-                if (bins_on && ti.p != tab_p) {
-                    // lay out the per-problem region for this problem: every thread is done
-                    // with the previous problem's bins (flushed and zeroed at each tile's end)
-                    // and table, then the new bins are zeroed and the new table loaded
-                    epi_sync(kEpiThreads);
-                    bins = reinterpret_cast<float *>(epi + EL.var);
-                    thr_s = reinterpret_cast<float *>(epi + EL.var + var_bins_bytes(E.NW, EW));
-                    for (int k = et; k < (E.NW + 1) * kBinStride; k += kEpiThreads) bins[k] = 0.f;
-                    // thresholds, or the lattice d2 -> bin table, of this problem
+            if (lane == 0 && got) mbar_arrive(wqempty0 + 8 * qs);
+            const bool end = got && p < 0;
+            const bool first = kci == 0, last = lst != 0;
+            if (got && !end && p != cur_p) {
+                // (a thread whose wait gave up meets the others at this barrier from the one
+                // below: it is the same barrier, and all stop)
+                ok = epi_sync_and(true, kEpiThreads);
+                if (!ok) break;
+                // another problem: finish the previous one, then load its parameters and
+                // lay out the per-problem region (every bin was zeroed at its flush)
+                if (cur_p >= 0) flush_acc(cur_p, cur_t);
+                epi_sync(kEpiThreads);
+                const uint32_t *src = reinterpret_cast<const uint32_t *>(&probs[p].epi);
+                uint32_t *dst = reinterpret_cast<uint32_t *>(epi + EL.par);
+                for (int k = et; k < (int)(sizeof(EpiParams) / 4); k += kEpiThreads)
+                    dst[k] = src[k];
+                epi_sync(kEpiThreads);
+                cur_p = p;
+                cur_t = t;
+                N = probs[p].dims.N;
+                det = E.fix_scale != nullptr;
+                fscale = det ? *E.fix_scale : 0.0;
+                if (!row_ok) ic = N - 1;
+                load_row();
+                bins = reinterpret_cast<float *>(epi + EL.var);
+                thr_s = reinterpret_cast<float *>(epi + EL.var + var_bins_bytes(E.NW, EW));
+                // (a checked build also tests that the problem's bins and table fit the
+                // launch's per-problem region; if not, the problem is not binned)
+                bins_on = E.n_bins > 0 &&
+                          ASD_INB(var_bytes(E.NW, E.n_bins, E.n_lut, EW) <= args.VB,
+                                  BND_REGION, args.err);
+                if (bins_on) {
+                    for (int k = et; k < (E.NW + 1) * kBinStride; k += kEpiThreads)
+                        bins[k] = 0.f;
                     if (E.n_lut > 0) {
-                        // fast form: entries become private-bin word offsets (the host checked
-                        // that (n_bins + 1) * stride fits 16 bits)
-                        // (dropped pairs: the trash row E.NW, which no flush reads)
+                        // fast form: entries become private-bin word offsets (the host
+                        // checked that (n_bins + 1) * stride fits 16 bits); dropped
+                        // pairs: the trash row E.NW, which no flush reads
                         uint16_t *lut_s = reinterpret_cast<uint16_t *>(thr_s);
                         for (int k = et; k < E.n_lut; k += kEpiThreads) {
                             const int b = E.lut[k];
-                            lut_s[k] = (uint16_t)(fast_ok(E) ? (b < E.n_bins ? b : E.NW) * kBinStride
-                                                             : b);
+                            lut_s[k] = (uint16_t)(fast_ok()
+                                                      ? (b < E.n_bins ? b : E.NW) * kBinStride
+                                                      : b);
                         }
                     } else {
                         float2 *thr2 = reinterpret_cast<float2 *>(thr_s);
                         for (int k = et; k <= E.n_bins; k += kEpiThreads)
                             thr2[k] = make_float2(E.thr[k], E.thr[k + 1]);
                     }
-                    tab_p = ti.p;
                 }
-                // column geometry of the tile (one load per column, which also feeds the
-                // column bounding box when the bins do not all fit the window)
-                float cl[3] = {3e38f, 3e38f, 3e38f}, ch[3] = {-3e38f, -3e38f, -3e38f};
-                // (and the box of each 32-column chunk this warp loads: chunk ew + m EW)
-                float cm[kColM][6];
-#pragma unroll
-                for (int m = 0; m < kColM; ++m)
-#pragma unroll
-                    for (int a = 0; a < 3; ++a) {
-                        cm[m][a] = 3e38f;
-                        cm[m][3 + a] = -3e38f;
-                    }
-#pragma unroll
-                for (int m = 0; m < kColM; ++m) {
-                    const int c = et + m * kEpiThreads;
-                    if (c >= BN) break;
-                    const int j = min(ti.n0 + c, P.N - 1);
-                    float4 pj;
-                    if (lattice) {
-                        const int4 g = E.coords[j];
-                        colgeo[c] = __int_as_float(g.x);
-                        colgeo[BN + c] = __int_as_float(g.y);
-                        colgeo[2 * BN + c] = __int_as_float(g.z);
-                        colpk[c] = (uint32_t)g.x | ((uint32_t)g.y << 8) | ((uint32_t)g.z << 16);
-                        pj = make_float4((float)g.x, (float)g.y, (float)g.z, 0.f);
-                    } else {
-                        pj = E.pos[j];
-                        colgeo[c] = pj.x;
-                        colgeo[BN + c] = pj.y;
-                        colgeo[2 * BN + c] = pj.z;
-                    }
-                    cl[0] = fminf(cl[0], pj.x); ch[0] = fmaxf(ch[0], pj.x);
-                    cl[1] = fminf(cl[1], pj.y); ch[1] = fmaxf(ch[1], pj.y);
-                    cl[2] = fminf(cl[2], pj.z); ch[2] = fmaxf(ch[2], pj.z);
-                    cm[m][0] = pj.x; cm[m][1] = pj.y; cm[m][2] = pj.z;
-                    cm[m][3] = pj.x; cm[m][4] = pj.y; cm[m][5] = pj.z;
+                epi_sync(kEpiThreads);
+            } else if (got && !end && first && t != cur_t) {
+                new_t = true;
+            }
+            if (got && !end) {
+                if (first)
+                    got = mbar_wait(gfull0 + 8 * (item & 1), (item >> 1) & 1, args.err,
+                                    DEV_TIMEOUT_EPI);
+                got = got && mbar_wait(tfull0 + 8 * acc, use & 1, args.err, DEV_TIMEOUT_EPI);
+            }
+            // (also orders the flush of the previous tile's private bins before new adds)
+            ok = epi_sync_and(got, kEpiThreads);
+            if (!ok || end) break;
+            tc_after();
+            if (first) {
+                if (new_t) {
+                    flush_acc(cur_p, cur_t);
+                    cur_t = t;
                 }
-                ri = E.coords[ic];
-                rp = lattice ? make_float4((float)ri.x, (float)ri.y, (float)ri.z, 0.f) : E.pos[ic];
-                // bounding boxes for the bin window (only when the bins do not all fit)
-                if (E.use_window) {
-                    float v6[12];
-                    v6[0] = v6[3] = rp.x;
-                    v6[1] = v6[4] = rp.y;
-                    v6[2] = v6[5] = rp.z;
-                    for (int a = 0; a < 3; ++a) {
-                        v6[6 + a] = cl[a];
-                        v6[9 + a] = ch[a];
-                    }
-                    if (!row_ok) {
-                        for (int a = 0; a < 3; ++a) {
-                            v6[a] = 3e38f;
-                            v6[3 + a] = -3e38f;
-                        }
-                    }
-                    for (int o = 16; o > 0; o >>= 1)
-                        for (int k = 0; k < 12; ++k) {
-                            const float w = __shfl_xor_sync(0xffffffffu, v6[k], o);
-                            v6[k] = ((k % 6) < 3) ? fminf(v6[k], w) : fmaxf(v6[k], w);
-                        }
-                    if (lane == 0)
-                        for (int k = 0; k < 12; ++k) boxred[ew * 12 + k] = v6[k];
-                    if (!lattice) {
-#pragma unroll
-                        for (int m = 0; m < kColM; ++m) {
-                            const int chk = ew + m * kEpiWarps;  // warp-uniform
-                            if (chk >= kChunks) break;
-                            for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-                                for (int k = 0; k < 6; ++k) {
-                                    const float w = __shfl_xor_sync(0xffffffffu, cm[m][k], o);
-                                    cm[m][k] = k < 3 ? fminf(cm[m][k], w) : fmaxf(cm[m][k], w);
-                                }
-                            if (lane == 0)
-#pragma unroll
-                                for (int k = 0; k < 6; ++k) chbox[chk * 6 + k] = cm[m][k];
-                        }
-                    }
-                }
-                epi_sync(kEpiThreads);  // colgeo / boxred ready; previous tile fully flushed
-                if (ti.p != cur_p || ti.t != cur_t) {
-                    if (cur_p >= 0) flush_acc(cur_p, cur_t);
-                    cur_p = ti.p;
-                    cur_t = ti.t;
-                }
-                blo = 0;
-                n1 = E.NW;
-                split = kChunks;
-                nwp = E.n_bins;
-                // positions: whether every kept bin of the tile lies inside the private window
-                // [blo, blo + NW), from the largest distance between the two bounding boxes
-                pos_fit = !E.use_window && E.pos_ok;
-                bhi_tile = E.n_bins - 1;
-                if (E.use_window) {
-                    float d2min = 0.f, d2max = 0.f;
-                    for (int a = 0; a < 3; ++a) {
-                        float rl = 3e38f, rh = -3e38f, cl = 3e38f, ch = -3e38f;
-                        for (int w = 0; w < kEpiWarps; ++w) {
-                            rl = fminf(rl, boxred[w * 12 + a]);
-                            rh = fmaxf(rh, boxred[w * 12 + 3 + a]);
-                            cl = fminf(cl, boxred[w * 12 + 6 + a]);
-                            ch = fmaxf(ch, boxred[w * 12 + 9 + a]);
-                        }
-                        float gap = fmaxf(0.f, fmaxf(cl - rh, rl - ch));
-                        if (lattice && E.periodic) {
-                            const float L = a == 0 ? E.Lx : a == 1 ? E.Ly : E.Lz;
-                            gap = fminf(gap, fmaxf(0.f, fmaxf(cl + L - rh, rl - (ch + L))));
-                            gap = fminf(gap, fmaxf(0.f, fmaxf(cl - L - rh, rl - (ch - L))));
-                        }
-                        d2min += gap * gap;
-                        const float far = fmaxf(ch - rl, rh - cl);
-                        d2max += far * far;
-                    }
-                    // (the thresholds from shared memory unless it holds the lattice table)
-                    const float2 *thr2 = reinterpret_cast<const float2 *>(thr_s);
-                    const bool tab = E.n_lut > 0;
-                    blo = max(0, (tab ? bin_of_d2(d2min * 0.999f, E.inv_w, E.n_bins, E.thr)
-                                      : bin_of_d2_pair(d2min * 0.999f, E.inv_w, E.n_bins, thr2,
-                                                       args.err)) - 1);
-                    if (!lattice) {
-                        bhi_tile = min(E.n_bins - 1,
-                                       bin_of_d2_pair(d2max * 1.001f + 1e-30f, E.inv_w, E.n_bins,
-                                                      thr2, args.err) + 1);
-                        pos_fit = E.pos_ok && bhi_tile - blo < E.NW;
-                        nwp = bhi_tile - blo + 1;
-                        if (!pos_fit && E.pos_ok) {
-                            // bins of each 32-column chunk (lane c computes chunk c), then the
-                            // first split of the chunks into two windows that together fit
-                            int lo_c = 1 << 30, hi_c = -1;
-                            if (lane < kChunks) {
-                                float dmin = 0.f, dmax = 0.f;
-                                for (int a = 0; a < 3; ++a) {
-                                    float rl = 3e38f, rh = -3e38f;
-                                    for (int w = 0; w < kEpiWarps; ++w) {
-                                        rl = fminf(rl, boxred[w * 12 + a]);
-                                        rh = fmaxf(rh, boxred[w * 12 + 3 + a]);
-                                    }
-                                    const float cl = chbox[lane * 6 + a], ch = chbox[lane * 6 + 3 + a];
-                                    const float gap = fmaxf(0.f, fmaxf(cl - rh, rl - ch));
-                                    const float far = fmaxf(ch - rl, rh - cl);
-                                    dmin += gap * gap;
-                                    dmax += far * far;
-                                }
-                                lo_c = max(0, bin_of_d2_pair(dmin * 0.999f, E.inv_w, E.n_bins, thr2,
-                                                             args.err) - 1);
-                                hi_c = min(E.n_bins - 1,
-                                           bin_of_d2_pair(dmax * 1.001f + 1e-30f, E.inv_w,
-                                                          E.n_bins, thr2, args.err) + 1);
-                            }
-                            int lo[kChunks], hi[kChunks];
-#pragma unroll
-                            for (int c = 0; c < kChunks; ++c) {
-                                lo[c] = __shfl_sync(0xffffffffu, lo_c, c);
-                                hi[c] = __shfl_sync(0xffffffffu, hi_c, c);
-                            }
-                            // one window over the chunks' bins (narrower than the tile's
-                            // box); only when that does not fit, two windows, which are then
-                            // disjoint (two overlapping ones would span no more than their
-                            // sum), so no bin has two private rows
-                            int l0 = 1 << 30, h0 = -1;
-#pragma unroll
-                            for (int c = 0; c < kChunks; ++c) {
-                                l0 = min(l0, lo[c]);
-                                h0 = max(h0, hi[c]);
-                            }
-                            int best = E.NW + 1;
-                            if (h0 - l0 + 1 <= E.NW) {
-                                best = h0 - l0 + 1;
-                                blo = l0;
-                                n1 = E.NW;
-                                split = kChunks;
-                            }
-#pragma unroll
-                            for (int sp = 1; sp < kChunks && best > E.NW; ++sp) {
-                                int l1 = 1 << 30, h1 = -1, l2 = 1 << 30, h2 = -1;
-#pragma unroll
-                                for (int c = 0; c < kChunks; ++c) {
-                                    if (c < sp) { l1 = min(l1, lo[c]); h1 = max(h1, hi[c]); }
-                                    else { l2 = min(l2, lo[c]); h2 = max(h2, hi[c]); }
-                                }
-                                const int need = (h1 - l1 + 1) + (h2 - l2 + 1);
-                                if (need < best) {
-                                    best = need;
-                                    blo = l1;
-                                    n1 = h1 - l1 + 1;
-                                    blo2 = l2;
-                                    split = sp;
-                                }
-                            }
-                            if (best <= E.NW) {
-                                pos_fit = true;
-                                nwp = best;
-                            } else {
-                                blo = max(0, (tab ? bin_of_d2(d2min * 0.999f, E.inv_w, E.n_bins, E.thr)
-                                                  : bin_of_d2_pair(d2min * 0.999f, E.inv_w, E.n_bins,
-                                                                   thr2, args.err)) - 1);
-                                n1 = E.NW;
-                                split = kChunks;
-                            }
-                        } else {
-                            n1 = E.NW;
-                            split = kChunks;
-                        }
-                    }
-                }
-            }  // first chunk
-
+                const uint32_t gb = item & 1;
+                colgeo = reinterpret_cast<const float *>(epi + EL.geo) + gb * 3 * BN;
+                tw = reinterpret_cast<const TileWindow *>(epi + EL.win)[gb];
+                ++item;
+            }
+            const bool lattice = E.geom == ASD_GEOM_LATTICE;
             // phase weights of this item go through the tensor core (see kPhaseOK)
             const bool ph = kPhaseOK && E.n_q > 0;
-            const uint32_t acc = v & 1, use = v >> 1;
-            const bool got = mbar_wait(tfull0 + 8 * acc, use & 1, args.err, DEV_TIMEOUT_EPI);
-            ok = epi_sync_and(got, kEpiThreads);
-            if (!ok) break;
-            tc_after();
             const uint32_t tbase = tmem + ((uint32_t)(q4 * 32) << 16) + acc * BN;
 
             if (bins_on) {
@@ -1659,7 +1889,7 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) pc_tc_kernel(const __grid_con
                 ba.periodic = E.periodic;
                 ba.inv_w = E.inv_w;
                 ba.nb = E.n_bins;
-                ba.blo = E.use_window ? blo : 0;
+                ba.blo = E.use_window ? tw.blo : 0;
                 ba.nwp = E.use_window ? E.NW : E.n_bins;
                 ba.trash = E.NW;
                 ba.NB = args.NB;
@@ -1667,7 +1897,7 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) pc_tc_kernel(const __grid_con
                 ba.fscale = fscale;
                 ba.err = args.err;
                 const int mode = !lattice ? BIN_POS : (E.n_lut > 0 ? BIN_LUT : BIN_THR);
-                if (fast_ok(E)) {
+                if (fast_ok()) {
                     // rows past the range skip the pairs (the TMEM loads stay warp-wide)
                     const uint32_t rpk =
                         (uint32_t)ri.x | ((uint32_t)ri.y << 8) | ((uint32_t)ri.z << 16);
@@ -1678,7 +1908,7 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) pc_tc_kernel(const __grid_con
                         // the TMEM load runs while the bin offsets are computed
                         uint32_t g[32], off[32];
                         tmem_ld32_issue(tbase + ch * 32, g);
-                        const uint4 *cp = reinterpret_cast<const uint4 *>(colpk + ch * 32);
+                        const uint4 *cp = reinterpret_cast<const uint4 *>(colgeo) + ch * 8;
                         if (lut)
                             pk_offsets<true, kBinStride>(off, rpk, E.Lpk, cp, thr_s, E.inv_w,
                                                          E.n_bins, trash_off, E.n_lut, args.err);
@@ -1689,7 +1919,7 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) pc_tc_kernel(const __grid_con
                         if (row_ok) add_private(mb, off, g, trash_off, args.err);
                         if (ph) to_bf16(g, tbase + ch * 32, row_ok);
                     }
-                } else if (mode == BIN_POS && pos_fit) {
+                } else if (mode == BIN_POS && tw.fit) {
                     // rows past the range skip the pairs (the TMEM loads stay warp-wide)
                     float *mb = bins + r + kBM * half;
                     const uint32_t trash_off = (uint32_t)E.NW * kBinStride;
@@ -1699,10 +1929,10 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) pc_tc_kernel(const __grid_con
                     const uint64_t nx = pack2(-rp.x, -rp.x), ny = pack2(-rp.y, -rp.y),
                                    nz = pack2(-rp.z, -rp.z);
                     // whether some pair of the tile may lie at n_bins or beyond
-                    const bool drop = !E.no_drop && (!E.use_window || bhi_tile == E.n_bins - 1);
+                    const bool drop = !E.no_drop && (!E.use_window || tw.bhi == E.n_bins - 1);
                     for (int ch = ch0; ch < ch1; ++ch) {
                         // (private row of bin b: b - blo, or b - blo2 + n1 in a second window)
-                        const int b0 = !E.use_window ? 0 : ch < split ? blo : blo2 - n1;
+                        const int b0 = !E.use_window ? 0 : ch < tw.split ? tw.blo : tw.blo2 - tw.n1;
                         uint32_t g[32], off[32];
                         tmem_ld32_issue(tbase + ch * 32, g);
                         const float *cg = colgeo + ch * 32;
@@ -1725,7 +1955,7 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) pc_tc_kernel(const __grid_con
                     tmem_ld32(tbase + ch * 32, g);
                     const float *cg = colgeo + ch * 32;
                     float *mb = bins + r + kBM * half;
-                    void *fbv = fscale != 0.0 ? static_cast<void *>(fbi) : static_cast<void *>(fb);
+                    void *fbv = det ? static_cast<void *>(fbi) : static_cast<void *>(fb);
                     if (mode == BIN_LUT)
                         bin_chunk<BIN_LUT, kBinStride>(g, row_ok, ri, rp, cg, BN, thr_s, mb, fbv,
                                                       ba);
@@ -1756,50 +1986,65 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) pc_tc_kernel(const __grid_con
                 if constexpr (CG == 2) mbar_arrive_cl(lead(a));
                 else mbar_arrive(a);
             }
+            // the tile's geometry buffer may be filled again
+            if (last && lane == 0) mbar_arrive(gempty0 + 8 * ((item - 1) & 1));
             if (last) epi_sync(kEpiThreads);  // all private bins written
             if (bins_on && last) {
                 // private rows this tile may have written: with the branch-free position
                 // path only the tile's own bin range, else the whole window / bin set
                 const int NWp = !E.use_window ? E.n_bins
-                                : (!lattice && pos_fit ? min(E.NW, nwp) : E.NW);
-                // epilogue warp ew reduces bins b = 4 ew + u (mod 4 EW), four at a time (the
-                // four shuffle trees overlap): conflict-free loads, an FP32 tree over the
-                // stride, one FP64 add per bin (the FP64 pipe is narrow on this part, so
-                // FP64 work is kept per bin, not per row)
-                for (int b0 = 4 * ew; b0 < NWp; b0 += 4 * kEpiWarps) {
-                    float v4[4];
+                                : (!lattice && tw.fit ? min(E.NW, tw.nwp) : E.NW);
+                // epilogue warp ew reduces eight bins at a time: conflict-free loads, then the
+                // FP32 tree of the warp by recursive halving (each exchange sends the half
+                // of the bins this lane does not keep: 9 shuffles for 8 bins), after which
+                // every fourth lane holds one of the bins.  Lane & 3 picks the round, so one
+                // FP64 conversion and add serves up to four rounds, 32 bins (the FP64 pipe
+                // is narrow on this part; one lane adding bin after bin took most of this
+                // part's time: 8.2 -> 2.7 thousand cycles per tile on a 34^3 lattice, 6.3 -> 3.5
+                // on the 32^3 glass).
+                for (int b0 = 8 * ew; b0 < NWp; b0 += 32 * kEpiWarps) {
+                    float sum = 0.f;
+                    int k = NWp;
+#pragma unroll 1
+                    for (int rd = 0; rd < 4; ++rd) {
+                        const int b1 = b0 + rd * 8 * kEpiWarps;
+                        if (b1 >= NWp) break;
+                        float v8[8];
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        v4[u] = 0.f;
-                        if (b0 + u < NWp) {
-                            float *row = bins + (b0 + u) * kBinStride;
+                        for (int u = 0; u < 8; ++u) {
+                            // (past the last row: that row again, a value no lane keeps)
+                            const float *row = bins + min(b1 + u, NWp - 1) * kBinStride;
+                            v8[u] = 0.f;
 #pragma unroll
-                            for (int m = 0; m < kBinStride / 32; ++m) {
-                                v4[u] += row[lane + 32 * m];
-                                row[lane + 32 * m] = 0.f;
-                            }
+                            for (int m = 0; m < kBinStride / 32; ++m) v8[u] += row[lane + 32 * m];
+                        }
+                        __syncwarp();
+#pragma unroll
+                        for (int u = 0; u < 8; ++u) {
+                            float4 *row = reinterpret_cast<float4 *>(bins + (b1 + u) * kBinStride);
+                            if (b1 + u < NWp)
+#pragma unroll
+                                for (int m = 0; m < kBinStride / 128; ++m)
+                                    row[lane + 32 * m] = make_float4(0.f, 0.f, 0.f, 0.f);
+                        }
+                        const float sr = warp_sum8(v8, lane);
+                        if ((lane & 3) == rd) {
+                            sum = sr;
+                            k = b1 + ((lane >> 4) & 1) * 4 + ((lane >> 3) & 1) * 2 +
+                                ((lane >> 2) & 1);
                         }
                     }
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-                        for (int u = 0; u < 4; ++u) v4[u] += __shfl_xor_sync(0xffffffffu, v4[u], o);
-                    if (lane == 0)
-#pragma unroll
-                        for (int u = 0; u < 4; ++u) {
-                            const int k = b0 + u;
-                            const int b = k < n1 ? blo + k : blo2 + (k - n1);
-                            if (k < NWp && b < E.n_bins &&
-                                ASD_INB(b < args.NB, BND_CACC, args.err)) {
-                                if (fscale != 0.0) cacci[b] += to_fixed((double)v4[u], fscale);
-                                else cacc[b] += (double)v4[u];
-                            }
-                        }
+                    const int b = k < tw.n1 ? tw.blo + k : tw.blo2 + (k - tw.n1);
+                    if (k < NWp && b < E.n_bins && ASD_INB(b < args.NB, BND_CACC, args.err)) {
+                        if (det) cacci[b] += to_fixed((double)sum, fscale);
+                        else cacc[b] += (double)sum;
+                    }
                 }
-                if (E.use_window) {
+                // (tiles whose bins all fit the window put nothing into the fallback bins)
+                if (E.use_window && (lattice || !tw.fit)) {
                     epi_sync(kEpiThreads);  // the fallback bins update the same accumulators
                     for (int b = et; b < E.n_bins; b += kEpiThreads) {
-                        if (fscale != 0.0) {
+                        if (det) {
                             cacci[b] += fbi[b];
                             fbi[b] = 0;
                         } else if (fb[b] != 0.f) {
@@ -1808,87 +2053,6 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) pc_tc_kernel(const __grid_con
                         }
                     }
                 }
-            }
-            // the phase product is read out once per pass; with one pass per tile P sums
-            // the tile's K chunks and is read out after the last
-            if (ph && (E.npass > 1 || last)) {
-                // Phase product of each pass: P[r][o] = sum_c G_rc W_co, u = P[.][0:64)
-                // (cosine column weights), v = P[.][64:128) (sine).  Row r adds
-                // cos(q.r_i) u + sin(q.r_i) v (cosine part) and sin(q.r_i) u - cos(q.r_i) v
-                // (sine part), the angle-difference identities of Eq. 6's weight; the warp
-                // then sums its 32 rows by recursive halving (each lane ends with one q
-                // of the 16) and adds it to the CTA's FP64 sums.
-                const float4 *cs4 = reinterpret_cast<const float4 *>(E.cs) +
-                                    (int64_t)ic * (E.nq_pad / 2);
-                const uint32_t pt = tmem + ((uint32_t)(q4 * 32) << 16) + 2 * BN;
-                // (with 8 epilogue warps the two warps of a lane quarter take half of
-                // the pass's q-vectors each)
-                constexpr int kJ = kPhaseQ / 16 / kHalves;
-                // row weights of 16 q-vectors (8 float4: cos, sin of two q each): the
-                // loads of the next group are in flight while the current one is used,
-                // those of a pass's first group while its product completes
-                auto load_cs = [&](float4 (&c)[8], int q0) {
-                    if (q0 < E.n_q && ASD_INB(q0 + 16 <= E.nq_pad, BND_Q, args.err))
-#pragma unroll
-                        for (int k = 0; k < 8; ++k) c[k] = cs4[q0 / 2 + k];
-                };
-                for (int pp = 0; pp < E.npass && ok; ++pp) {
-                    float4 c4[8];
-                    load_cs(c4, pp * kPhaseQ + 16 * half * kJ);
-                    const bool gotp = mbar_wait(pfull, n_pass & 1, args.err, DEV_TIMEOUT_EPI);
-                    ++n_pass;
-                    ok = epi_sync_and(gotp, kEpiThreads);
-                    if (!ok) break;
-                    tc_after();
-                    for (int j = half * kJ; j < (half + 1) * kJ; ++j) {
-                        const int q0 = pp * kPhaseQ + 16 * j;
-                        if (q0 >= E.n_q) break;
-                        uint32_t u[16], w[16];
-                        if (j > half * kJ) load_cs(c4, q0);
-                        tmem_ld16(pt + 16 * j, u);
-                        tmem_ld16(pt + kPhaseQ + 16 * j, w);
-                        tmem_wait16x2(u, w);
-                        float x[16], y[16];
-#pragma unroll
-                        for (int k = 0; k < 8; ++k) {
-                            const float ca = c4[k].x, sa = c4[k].y, cb = c4[k].z, sb = c4[k].w;
-                            const float u0 = __uint_as_float(u[2 * k]), v0 = __uint_as_float(w[2 * k]);
-                            const float u1 = __uint_as_float(u[2 * k + 1]);
-                            const float v1 = __uint_as_float(w[2 * k + 1]);
-                            x[2 * k] = fmaf(ca, u0, sa * v0);
-                            x[2 * k + 1] = fmaf(cb, u1, sb * v1);
-                            y[2 * k] = fmaf(sa, u0, -ca * v0);
-                            y[2 * k + 1] = fmaf(sb, u1, -cb * v1);
-                        }
-                        const int qme = q0 + (lane >> 1);
-                        const bool qok = (lane & 1) == 0 && qme < E.n_q &&
-                                         ASD_INB(qme < args.NQ, BND_Q, args.err);
-                        // deterministic mode: fixed-point adds (any order, same bits)
-                        const float xs = warp_sum16(x, lane);
-                        if (qok) {
-                            if (fscale != 0.0)
-                                add_fixed(&qacci[2 * qme], to_fixed((double)xs, fscale));
-                            else atomicAdd(&qacc[2 * qme], (double)xs);
-                        }
-                        if (E.q_parts == 2) {
-                            const float ys = warp_sum16(y, lane);
-                            if (qok) {
-                                if (fscale != 0.0)
-                                    add_fixed(&qacci[2 * qme + 1], to_fixed((double)ys, fscale));
-                                else
-                                    atomicAdd(&qacc[2 * qme + 1], (double)ys);
-                            }
-                        }
-                    }
-                    // P read: the next pass (or item) may overwrite it
-                    tc_before();
-                    __syncwarp();
-                    if (lane == 0) {
-                        if constexpr (CG == 2) mbar_arrive_cl(lead(pempty));
-                        else mbar_arrive(pempty);
-                    }
-                }
-                if (!ok) break;
             }
         }
         epi_sync(kEpiThreads);
@@ -1903,13 +2067,20 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) pc_tc_kernel(const __grid_con
         tc_after();
         tmem_dealloc<CG>(tmem, kTmemAlloc);
     }
+    // the last CTA to finish leaves the work-item counter at zero for the next launch (a
+    // memset before every launch cost a small call 1.5 us); every claim was made before
+    if (CG == 1 && args.counter && threadIdx.x == 0 &&
+        atomicAdd(args.counter + 1, 1ull) == gridDim.x - 1) {
+        args.counter[0] = 0;
+        args.counter[1] = 0;
+    }
 }
 
 template <int FORM, int BN, int SWB, int EW, int CG>
 int launch_one(const LaunchArgs &a, size_t smem, int sm_count, cudaStream_t s)
 {
     auto k = pc_tc_kernel<FORM, BN, SWB, EW, CG>;
-    constexpr int kThreads = 64 + 32 * EW;
+    constexpr int kThreads = tc_threads(BN, EW);
     ASD_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     if constexpr (CG == 1) {
         // persistent: one CTA per SM, no more CTAs than work items

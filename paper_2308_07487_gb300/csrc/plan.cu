@@ -147,6 +147,8 @@ static EpiParams epi_of(const asd_corr_plan *p)
     e.npass = p->tc && p->n_q > 0 ? (p->n_q + kPhaseQ - 1) / kPhaseQ : 0;
     e.q_parts = p->q_parts;
     e.cs = p->cs;
+    e.csT = p->csT;
+    e.cs_ld = p->N;
     e.C_fix = p->C_fix;
     e.Sq_fix = p->Sq_fix;
     e.fix_scale = p->d.deterministic ? p->fix_scale : nullptr;
@@ -248,21 +250,23 @@ static int fill_problem(asd_corr_plan *p, TcProblem *tp, int64_t row_begin, int6
             if (rc) return rc;
         }
     }
-    tp->N = (int)p->N;
-    tp->row_begin = (int)row_begin;
-    tp->row_end = (int)row_end;
-    tp->tiles_m = (int)((row_end - row_begin + kBM * p->CG - 1) / (kBM * p->CG));
-    tp->tiles_n = (int)((p->N + p->BN - 1) / p->BN);
-    tp->n_t = p->n_t;
-    tp->S = p->S;
-    tp->F3 = 3 * p->F;
-    tp->Kseg = (int)p->Kseg;
-    tp->nkb = (int)(p->Kseg / p->BK);
-    tp->n_copies = p->n_copies;
-    tp->group_m = p->d.raster_m > 0 ? p->d.raster_m : 16;
-    tp->k_chunks = p->k_chunks;
-    tp->n_tiles = tc_work_items(p->n_t, tp->tiles_m, tp->tiles_n);
+    TcDims &d = tp->dims;
+    d.N = (int)p->N;
+    d.row_begin = (int)row_begin;
+    d.row_end = (int)row_end;
+    d.tiles_m = (int)((row_end - row_begin + kBM * p->CG - 1) / (kBM * p->CG));
+    d.tiles_n = (int)((p->N + p->BN - 1) / p->BN);
+    d.n_t = p->n_t;
+    d.S = p->S;
+    d.F3 = 3 * p->F;
+    d.Kseg = (int)p->Kseg;
+    d.nkb = (int)(p->Kseg / p->BK);
+    d.n_copies = p->n_copies;
+    d.group_m = p->d.raster_m > 0 ? p->d.raster_m : 16;
+    d.k_chunks = p->k_chunks;
+    tp->n_tiles = tc_work_items(p->n_t, d.tiles_m, d.tiles_n);
     tp->epi = epi_of(p);
+    d.npass = tp->epi.npass;
     return ASD_OK;
 }
 
@@ -372,6 +376,7 @@ void asd_pair_corr_plan_destroy(asd_corr_plan *p)
     cudaFree(p->thr);
     cudaFree(p->lut);
     cudaFree(p->cs);
+    cudaFree(p->csT);
     cudaFree(p->W);
     cudaFree(p->sqF);
     cudaFree(p->counter);
@@ -679,6 +684,7 @@ int asd_pair_corr_plan_create(const asd_corr_desc *d, asd_corr_plan **out)
             // rows padded with zeros to whole q-chunks (aligned float4 loads, no tail)
             const int nqp = (p->n_q + kQChunk - 1) / kQChunk * kQChunk;
             std::vector<float2> cs((size_t)p->N * nqp, make_float2(0.f, 0.f));
+            std::vector<double> xs(tc ? 2 * (size_t)p->N * p->n_q : 0);  // (cos, sin) in FP64
             for (int64_t i = 0; i < p->N; ++i) {
                 double r[3];
                 for (int a = 0; a < 3; ++a)
@@ -686,7 +692,12 @@ int asd_pair_corr_plan_create(const asd_corr_desc *d, asd_corr_plan **out)
                                                            : (double)d->pos[3 * i + a];
                 for (int q = 0; q < p->n_q; ++q) {
                     double ph = d->q[3 * q] * r[0] + d->q[3 * q + 1] * r[1] + d->q[3 * q + 2] * r[2];
-                    cs[(size_t)i * nqp + q] = make_float2((float)cos(ph), (float)sin(ph));
+                    const double x[2] = {cos(ph), sin(ph)};
+                    cs[(size_t)i * nqp + q] = make_float2((float)x[0], (float)x[1]);
+                    if (tc) {
+                        xs[2 * ((size_t)i * p->n_q + q)] = x[0];
+                        xs[2 * ((size_t)i * p->n_q + q) + 1] = x[1];
+                    }
                 }
             }
             if (cudaMalloc(&p->cs, sizeof(float2) * cs.size()) != cudaSuccess) {
@@ -704,15 +715,11 @@ int asd_pair_corr_plan_create(const asd_corr_desc *d, asd_corr_plan **out)
                 p->Wld = (p->N + 7) / 8 * 8;
                 const size_t rows = (size_t)npass * 2 * kPhaseQ, plane = rows * p->Wld;
                 std::vector<uint16_t> W(2 * plane, 0);
+                std::vector<float2> csT((size_t)nqp * p->N, make_float2(0.f, 0.f));
                 for (int64_t c = 0; c < p->N; ++c) {
-                    double r[3];
-                    for (int a = 0; a < 3; ++a)
-                        r[a] = d->geometry == ASD_GEOM_LATTICE ? (double)d->coords[3 * c + a]
-                                                               : (double)d->pos[3 * c + a];
                     for (int q = 0; q < p->n_q; ++q) {
-                        const double ph = d->q[3 * q] * r[0] + d->q[3 * q + 1] * r[1] +
-                                          d->q[3 * q + 2] * r[2];
-                        const double x2[2] = {cos(ph), sin(ph)};
+                        const double *x2 = &xs[2 * ((size_t)c * p->n_q + q)];
+                        csT[(size_t)q * p->N + c] = cs[(size_t)c * nqp + q];
                         for (int part = 0; part < 2; ++part) {
                             const size_t row = (size_t)(q / kPhaseQ) * 2 * kPhaseQ +
                                                part * kPhaseQ + q % kPhaseQ;
@@ -723,6 +730,13 @@ int asd_pair_corr_plan_create(const asd_corr_desc *d, asd_corr_plan **out)
                         }
                     }
                 }
+                if (cudaMalloc(&p->csT, sizeof(float2) * csT.size()) != cudaSuccess) {
+                    cudaGetLastError();
+                    return fail(ASD_ENOMEM);
+                }
+                if (cudaMemcpy(p->csT, csT.data(), sizeof(float2) * csT.size(),
+                               cudaMemcpyHostToDevice))
+                    return fail(ASD_ECUDA);
                 if (cudaMalloc(&p->W, sizeof(uint16_t) * W.size()) != cudaSuccess) {
                     cudaGetLastError();
                     return fail(ASD_ENOMEM);
@@ -790,10 +804,12 @@ int asd_pair_corr_plan_create(const asd_corr_desc *d, asd_corr_plan **out)
     if (tc) {
         p->h_prob = new (std::nothrow) TcProblem;
         if (!p->h_prob || cudaMalloc(&p->d_prob, sizeof(TcProblem)) != cudaSuccess ||
-            cudaMalloc(&p->counter, sizeof(unsigned long long)) != cudaSuccess) {
+            cudaMalloc(&p->counter, 2 * sizeof(unsigned long long)) != cudaSuccess) {
             cudaGetLastError();
             return fail(ASD_ENOMEM);
         }
+        if (cudaMemset(p->counter, 0, 2 * sizeof(unsigned long long)) != cudaSuccess)
+            return fail(ASD_ECUDA);
         rc = fill_problem(p, p->h_prob, 0, p->N);
         if (rc) return fail(rc);
         if (cudaMemcpy(p->d_prob, p->h_prob, sizeof(TcProblem), cudaMemcpyHostToDevice) !=
@@ -868,12 +884,12 @@ int asd_pair_corr_contract_range(asd_corr_plan *p, int64_t row_begin, int64_t ro
     ov.t_begin = t_begin;
     ov.n_t = t_end - t_begin;
     ov.tiles_m = (int)((row_end - row_begin + kBM * p->CG - 1) / (kBM * p->CG));
-    ov.n_tiles = tc_work_items(ov.n_t, ov.tiles_m, p->h_prob->tiles_n);
+    ov.n_tiles = tc_work_items(ov.n_t, ov.tiles_m, p->h_prob->dims.tiles_n);
     ov.C_sum = C_sum;
     ov.Sq_sum = Sq_sum;
-    rc = launch_tc(p->d_prob, 1, ov.n_tiles, ov, p->prec, p->BN, p->swizzle_bytes, p->stages,
+    rc = launch_tc(p->d_prob, 1, p->h_prob->dims, ov.n_tiles, ov, p->prec, p->BN, p->swizzle_bytes, p->stages,
                    p->smem_bytes, tc_var_bytes(p->NW, p->n_bins, p->n_lut, p->EW), p->n_bins,
-                   p->n_q, p->EW, p->d.deterministic, p->CG, p->sm_count,
+                   p->n_q * p->q_parts, p->EW, p->d.deterministic, p->CG, p->sm_count,
                    p->d.static_schedule || p->CG == 2 ? nullptr : p->counter, s);
     return rc ? rc : fix_end(p, t_begin, t_end, C_sum, Sq_sum, s);
 }
@@ -898,7 +914,7 @@ int asd_pair_corr_batched(asd_corr_plan *const *plans, const float *const *trajs
         ASD_CHECK_ARG(p->n_bins == 0 || (C_sum && C_sum[k]), "C_sum required");
         ASD_CHECK_ARG(p->n_q == 0 || (Sq_sum && Sq_sum[k]), "Sq_sum required");
         ASD_CHECK_ARG(((uintptr_t)trajs[k] & 15) == 0, "traj must be 16-byte aligned");
-        max_nq = p->n_q > max_nq ? p->n_q : max_nq;
+        max_nq = p->n_q * p->q_parts > max_nq ? p->n_q * p->q_parts : max_nq;
         max_nb = p->n_bins > max_nb ? p->n_bins : max_nb;
     }
     // one smem configuration for the whole batch: the fixed epilogue arrays for the
@@ -951,7 +967,10 @@ int asd_pair_corr_batched(asd_corr_plan *const *plans, const float *const *trajs
             return ASD_ENOMEM;
         }
         owner->batch_last = new (std::nothrow) std::vector<TcProblem>();
-        if (!owner->batch_last) {
+        if (!owner->batch_last ||
+            cudaMemset(owner->batch_desc + kMaxProblems, 0, 256) != cudaSuccess) {
+            delete owner->batch_last;
+            owner->batch_last = nullptr;
             cudaFree(owner->batch_desc);
             owner->batch_desc = nullptr;
             return ASD_ENOMEM;
@@ -968,7 +987,7 @@ int asd_pair_corr_batched(asd_corr_plan *const *plans, const float *const *trajs
     auto items = [&](int k) {
         const asd_corr_plan *p = plans[k];
         return p->k_chunks *
-               tc_work_items(p->n_t, (int)((p->N + kBM - 1) / kBM), p->h_prob->tiles_n);
+               tc_work_items(p->n_t, (int)((p->N + kBM - 1) / kBM), p->h_prob->dims.tiles_n);
     };
     std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return items(a) > items(b); });
     std::vector<TcProblem> h((size_t)n);
@@ -978,10 +997,10 @@ int asd_pair_corr_batched(asd_corr_plan *const *plans, const float *const *trajs
         const asd_corr_plan *p = plans[k];
         TcProblem &hk = h[pos];
         hk = *p->h_prob;
-        hk.row_begin = 0;
-        hk.row_end = (int)p->N;
-        hk.tiles_m = (int)((p->N + kBM - 1) / kBM);
-        hk.n_tiles = tc_work_items(p->n_t, hk.tiles_m, hk.tiles_n);
+        hk.dims.row_begin = 0;
+        hk.dims.row_end = (int)p->N;
+        hk.dims.tiles_m = (int)((p->N + kBM - 1) / kBM);
+        hk.n_tiles = tc_work_items(p->n_t, hk.dims.tiles_m, hk.dims.tiles_n);
         hk.tile_begin = total;
         hk.epi.n_lut = nlut[k];  // 0: the threshold rule (see above)
         hk.epi.C_sum = C_sum ? C_sum[k] : nullptr;
@@ -1007,7 +1026,7 @@ int asd_pair_corr_batched(asd_corr_plan *const *plans, const float *const *trajs
     bool dyn = true;
     for (int k = 0; k < n; ++k) dyn = dyn && !plans[k]->d.static_schedule;
     unsigned long long *ctr = reinterpret_cast<unsigned long long *>(dbuf + kMaxProblems);
-    int rc = launch_tc(dbuf, n, total, ov, p0->prec, p0->BN, p0->swizzle_bytes, stages, smem, vb,
+    int rc = launch_tc(dbuf, n, h[0].dims, total, ov, p0->prec, p0->BN, p0->swizzle_bytes, stages, smem, vb,
                        max_nb, max_nq, p0->EW, p0->d.deterministic, 1, p0->sm_count,
                        dyn ? ctr : nullptr, s);
     for (int k = 0; k < n && !rc; ++k)
