@@ -9,9 +9,17 @@
 // in separate arrays so sites never race (Section 3.1).  No renormalisation: the paper
 // notes its RK4 evolution is not norm preserving.
 //
-// Each RK4 stage is one launch over (sample, site) -- a stage needs every neighbour's
-// previous stage.  The last stage writes the new state and, every `stride` steps, the
-// trajectory frame in the site-major layout traj[i][s][f][a] consumed by asd_pair_corr.
+// A stage needs every neighbour's previous stage.  Routes, by size (ll_run):
+//   ll_persistent<LOCAL>   one block per sample, the state in shared memory, a block barrier
+//                          between stages: samples of up to 2048 sites;
+//   ll_persistent<global>  a cooperative launch over every (sample, site), the state in L2,
+//                          a grid barrier between stages: up to four sites per thread;
+//   rk4_stage              one launch per stage: larger systems.
+// The last stage writes the new state and, every `stride` steps, the trajectory frame in the
+// site-major layout traj[i][s][f][a] consumed by asd_pair_corr.  All routes do the same
+// arithmetic in the same order.
+#include <algorithm>
+
 #include "asd_internal.h"
 
 namespace asd {
@@ -28,6 +36,22 @@ struct LLArgs {
     float A;
 };
 
+// One neighbour's part of the local field: J S_j, and D_ij x S_j with DM vectors (d: the
+// directed bond's, or null).
+__device__ __forceinline__ void add_bond(float3 &h, float J, float sx, float sy, float sz,
+                                         const float *__restrict__ d)
+{
+    h.x = fmaf(J, sx, h.x);
+    h.y = fmaf(J, sy, h.y);
+    h.z = fmaf(J, sz, h.z);
+    if (d) {
+        const float dx = __ldg(d), dy = __ldg(d + 1), dz = __ldg(d + 2);
+        h.x += dy * sz - dz * sy;
+        h.y += dz * sx - dx * sz;
+        h.z += dx * sy - dy * sx;
+    }
+}
+
 __device__ __forceinline__ float3 field(const LLArgs &a, const float *__restrict__ Y, int s,
                                         int64_t i)
 {
@@ -36,19 +60,8 @@ __device__ __forceinline__ float3 field(const LLArgs &a, const float *__restrict
     for (int k = 0; k < a.z; ++k) {
         const int j = __ldg(a.nbr + i * a.z + k);
         if (j < 0) continue;
-        const float Jij = __ldg(a.J + i * a.z + k);
-        h.x = fmaf(Jij, Ys[3 * (int64_t)j + 0], h.x);
-        h.y = fmaf(Jij, Ys[3 * (int64_t)j + 1], h.y);
-        h.z = fmaf(Jij, Ys[3 * (int64_t)j + 2], h.z);
-        if (a.D) {  // D_ij x S_j
-            const float *d = a.D + (i * a.z + k) * 3;
-            const float dx = __ldg(d), dy = __ldg(d + 1), dz = __ldg(d + 2);
-            const float sx = Ys[3 * (int64_t)j], sy = Ys[3 * (int64_t)j + 1],
-                        sz = Ys[3 * (int64_t)j + 2];
-            h.x += dy * sz - dz * sy;
-            h.y += dz * sx - dx * sz;
-            h.z += dx * sy - dy * sx;
-        }
+        add_bond(h, __ldg(a.J + i * a.z + k), Ys[3 * (int64_t)j], Ys[3 * (int64_t)j + 1],
+                 Ys[3 * (int64_t)j + 2], a.D ? a.D + (i * a.z + k) * 3 : nullptr);
     }
     h.z = fmaf(-2.f * a.A, Ys[3 * i + 2], h.z);
     return h;
@@ -108,6 +121,404 @@ __global__ void write_frame0(const float *__restrict__ Y, int64_t N, int S, floa
     dst[0] = src[0]; dst[1] = src[1]; dst[2] = src[2];
 }
 
+// ---------------------------------------------------------------------------------------
+// Persistent routes
+// ---------------------------------------------------------------------------------------
+constexpr int kLLThreads = 1024;
+constexpr int kLLMaxSpt = 4;                       // sites per thread
+constexpr size_t kLLMaxSmem = 220 * 1024;
+constexpr int kLLStepsPerLaunch = 4096;            // other streams' work gets in between
+constexpr unsigned long long kLLTimeoutNs = 4000000000ull;
+
+struct LLRun {
+    LLArgs a;
+    const float *in;     // [S][N][3] state at the first step
+    float *out;          // [S][N][3] state after the last step, or null
+    float4 *Y, *T1, *T2; // global route: state and stage inputs [S][N]
+    unsigned *bar;       // global route: grid barrier count (zero at launch)
+    float *traj;
+    int F;
+    int64_t step0, step1;  // steps [step0, step1) of the run
+    int stride;
+    float dt;
+    int stage_frames;    // 1: frames go out through shared memory, kLLFrames at a time
+    int *err;
+};
+constexpr int kLLFrames = 4;
+constexpr int kLLFramePitch = 3 * kLLFrames + 1;   // words per site (odd: no bank conflicts)
+
+// Barrier over all blocks of a cooperative launch: the count reaches `target` once every
+// block has arrived.  The release before the arrival and the acquire after the wait order
+// all blocks' global stores and loads around it (the acquire also drops this SM's L1 lines).
+// Bounded: false for every thread of the block after kLLTimeoutNs.
+__device__ __forceinline__ bool grid_barrier(unsigned *bar, unsigned target, int *err)
+{
+    __syncthreads();
+    int ok = 1;
+    if (threadIdx.x == 0) {
+        __threadfence();
+        asm volatile("red.relaxed.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
+        unsigned long long t0 = 0;
+        for (unsigned it = 0;; ++it) {
+            unsigned v;
+            asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
+            if ((int)(v - target) >= 0) break;
+            if ((it & 1023u) == 1023u) {
+                unsigned long long now;
+                asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
+                if (t0 == 0) t0 = now;
+                else if (now - t0 > kLLTimeoutNs) {
+                    atomicCAS(err, 0, (int)DEV_TIMEOUT_LL);
+                    ok = 0;
+                    break;
+                }
+            }
+        }
+        __threadfence();
+    }
+    return __syncthreads_and(ok) != 0;
+}
+
+// All steps of a launch.  Bound by the latency of a stage (380 to 640 dependent stages, each
+// a few hundred cycles of loads and arithmetic), not by bandwidth, so the work is to take the
+// launches, the index loads and the global round trips out of a stage: bonds (neighbour,
+// coupling) are read once, into registers for Z = 4 or 6 bonds and one site a thread, else
+// into shared memory (Z = 0: any number of bonds); state and derivative sum of the own sites stay in
+// registers; neighbours are read as one 16-byte word from shared memory (LOCAL) or L2.
+// Measured against a launch per stage: 50 samples of 16^2 sites, 95 steps, 1572 -> 121 us
+// (4.1 -> 0.32 us per stage); 64^3, 159 steps, 6.14 -> 3.36 ms (9.6 -> 5.3 us per stage, of
+// which the barrier about 2); frames stored by each site as they come instead of gathered:
+// 130 us and 3.78 ms.  36^2 sites and two samples, 90 steps: 1.58 -> 0.53 ms, though only
+// two blocks run (the grid route's stage takes 2.4 us at any size up to 50 thousand sites).
+template <int SPT, int Z, bool LOCAL>
+__global__ void __launch_bounds__(kLLThreads, 1) ll_persistent(const __grid_constant__ LLRun r)
+{
+    extern __shared__ __align__(16) uint8_t ll_smem[];
+    constexpr bool kReg = Z > 0 && SPT == 1;   // bonds in registers
+    const LLArgs &a = r.a;
+    const int N = (int)a.N, nt = blockDim.x, tid = threadIdx.x;
+    const int64_t n = (int64_t)N * a.S;
+    // LOCAL: block = sample, site = tid + k nt.  Else sites of the flattened (sample, site)
+    // list in contiguous runs of SPT nt per block.
+    const int64_t g0 = LOCAL ? (int64_t)blockIdx.x * N : (int64_t)blockIdx.x * SPT * nt;
+    // state arrays indexed by the flattened site minus `base`
+    const int64_t base = LOCAL ? g0 : 0;
+    float4 *Y = LOCAL ? reinterpret_cast<float4 *>(ll_smem) : r.Y;
+    float4 *T1 = LOCAL ? Y + N : r.T1;
+    float4 *T2 = LOCAL ? T1 + N : r.T2;
+    // bonds in shared memory: [k][slot], slot = site index within the block
+    int *sm_nbr = reinterpret_cast<int *>(ll_smem + (LOCAL ? (size_t)48 * N : 0));
+    const int slots = LOCAL ? N : SPT * nt;
+    float *sm_J = reinterpret_cast<float *>(sm_nbr + (kReg ? 0 : (size_t)a.z * slots));
+    float *sm_frames = sm_J + (kReg ? 0 : (size_t)a.z * slots);
+
+    constexpr int ZR = Z > 0 ? Z : 1, ZB = kReg ? Z : 1;
+    int nb[ZB];
+    float Jr[ZB];
+    float3 y[SPT], acc[SPT], x[SPT];
+    bool on[SPT];
+    int own[SPT];                      // index of the own site in the state arrays
+    int site[SPT];                     // site in its sample
+    float *dst[SPT];                   // its last trajectory frame
+#pragma unroll
+    for (int u = 0; u < SPT; ++u) {
+        const int slot = u * nt + tid;
+        const int64_t g = g0 + slot;
+        on[u] = LOCAL ? slot < N : g < n;
+        const int64_t gc = on[u] ? g : g0;
+        const int s = LOCAL ? (int)blockIdx.x : (int)(gc / N);
+        site[u] = (int)(gc - (int64_t)s * N);
+        const int off = (int)((int64_t)s * N - base);   // the sample's first index
+        own[u] = (int)(gc - base);
+        if (kReg) {
+#pragma unroll
+            for (int k = 0; k < ZB; ++k) {
+                const int j = on[u] ? __ldg(a.nbr + (int64_t)site[u] * Z + k) : -1;
+                nb[k] = j < 0 ? -1 : j + off;
+                Jr[k] = on[u] ? __ldg(a.J + (int64_t)site[u] * Z + k) : 0.f;
+            }
+        } else if (on[u]) {
+            for (int k = 0; k < a.z; ++k) {
+                const int j = __ldg(a.nbr + (int64_t)site[u] * a.z + k);
+                sm_nbr[k * slots + slot] = j < 0 ? -1 : j + off;
+                sm_J[k * slots + slot] = __ldg(a.J + (int64_t)site[u] * a.z + k);
+            }
+        }
+        const float *src = r.in + 3 * gc;
+        y[u] = make_float3(src[0], src[1], src[2]);
+        x[u] = y[u];
+        dst[u] = r.traj + (((int64_t)site[u] * a.S + s) * r.F + r.step0 / r.stride) * 3;
+        if (on[u]) {
+            Y[own[u]] = make_float4(y[u].x, y[u].y, y[u].z, 0.f);
+            if (r.step0 == 0) {
+                dst[u][0] = y[u].x; dst[u][1] = y[u].y; dst[u][2] = y[u].z;
+            }
+        }
+    }
+    int in_frame = (int)(r.step0 % r.stride);   // steps since the last frame
+    // Frames.  A frame's 12 bytes per site lie a trajectory row apart, so a warp storing one
+    // touches 32 lines per instruction; kLLFrames frames gathered in shared memory go out
+    // with consecutive lanes on consecutive words of a site's row.
+    int n_held = 0;
+    int64_t f_held = r.step0 / r.stride + 1;    // first frame held
+    auto put_frames = [&]() {
+        __syncthreads();   // every site's frames are in
+        const int words = 3 * n_held, left = LOCAL ? N : (int)min((int64_t)slots, n - g0);
+        for (int e = tid; e < left * words; e += nt) {
+            const int slot = e / words, c = e - slot * words;
+            const int64_t g = g0 + slot;
+            const int64_t s = LOCAL ? blockIdx.x : g / N, i = g - s * N;
+            r.traj[((i * a.S + s) * r.F + f_held) * 3 + c] = sm_frames[slot * kLLFramePitch + c];
+        }
+        f_held += n_held;
+        n_held = 0;
+        __syncthreads();   // the buffer may be filled again
+    };
+    unsigned target = 0;
+    auto barrier = [&]() {
+        if (LOCAL) {
+            __syncthreads();
+            return true;
+        }
+        target += gridDim.x;
+        return grid_barrier(r.bar, target, r.err);
+    };
+    if (!barrier()) return;
+
+    // derivative of own site u from the stage input V (own value x[u])
+    auto deriv = [&](int u, const float4 *V) {
+        float3 h = make_float3(0.f, 0.f, -a.Hz);
+        const int slot = u * nt + tid;
+        if (Z > 0) {
+            // all neighbours' loads in flight, then the sums in bond order
+            float4 sj[ZR];
+            int j[ZR];
+#pragma unroll
+            for (int k = 0; k < ZR; ++k) {
+                j[k] = kReg ? nb[kReg ? k : 0] : sm_nbr[k * slots + slot];
+                sj[k] = V[j[k] < 0 ? own[u] : j[k]];
+            }
+#pragma unroll
+            for (int k = 0; k < ZR; ++k)
+                if (j[k] >= 0)
+                    add_bond(h, kReg ? Jr[kReg ? k : 0] : sm_J[k * slots + slot], sj[k].x,
+                             sj[k].y, sj[k].z,
+                             a.D ? a.D + ((int64_t)site[u] * Z + k) * 3 : nullptr);
+        } else {
+            for (int k = 0; k < a.z; ++k) {
+                const int j = sm_nbr[k * slots + slot];
+                if (j < 0) continue;
+                const float4 sj = V[j];
+                add_bond(h, sm_J[k * slots + slot], sj.x, sj.y, sj.z,
+                         a.D ? a.D + ((int64_t)site[u] * a.z + k) * 3 : nullptr);
+            }
+        }
+        h.z = fmaf(-2.f * a.A, x[u].z, h.z);
+        return cross(h, x[u]);
+    };
+    for (int64_t st = r.step0; st < r.step1; ++st) {
+#pragma unroll
+        for (int stage = 1; stage <= 4; ++stage) {
+            const float4 *in = stage == 1 ? Y : stage == 3 ? T2 : T1;
+            float4 *out = stage == 4 ? Y : stage == 2 ? T2 : T1;
+#pragma unroll
+            for (int u = 0; u < SPT; ++u) {
+                if (!on[u]) continue;
+                const float3 k = deriv(u, in);
+                if (stage == 1) {
+                    acc[u] = k;
+                } else if (stage < 4) {
+                    acc[u].x += 2.f * k.x;
+                    acc[u].y += 2.f * k.y;
+                    acc[u].z += 2.f * k.z;
+                }
+                if (stage < 4) {
+                    const float c = stage == 3 ? r.dt : 0.5f * r.dt;
+                    x[u] = make_float3(fmaf(c, k.x, y[u].x), fmaf(c, k.y, y[u].y),
+                                       fmaf(c, k.z, y[u].z));
+                } else {
+                    const float c = r.dt / 6.f;
+                    y[u] = make_float3(fmaf(c, acc[u].x + k.x, y[u].x),
+                                       fmaf(c, acc[u].y + k.y, y[u].y),
+                                       fmaf(c, acc[u].z + k.z, y[u].z));
+                    x[u] = y[u];
+                }
+                out[own[u]] = make_float4(x[u].x, x[u].y, x[u].z, 0.f);
+            }
+            // (the frame's stores are in flight while the barrier runs)
+            if (stage == 4 && ++in_frame == r.stride) {
+                in_frame = 0;
+#pragma unroll
+                for (int u = 0; u < SPT; ++u) {
+                    dst[u] += 3;
+                    float *d = r.stage_frames
+                                   ? sm_frames + (u * nt + tid) * kLLFramePitch + 3 * n_held
+                                   : dst[u];
+                    if (on[u]) {
+                        d[0] = y[u].x; d[1] = y[u].y; d[2] = y[u].z;
+                    }
+                }
+                if (r.stage_frames && ++n_held == kLLFrames) put_frames();
+            }
+            if (!barrier()) return;
+        }
+    }
+    if (n_held > 0) put_frames();
+    if (r.out)
+#pragma unroll
+        for (int u = 0; u < SPT; ++u)
+            if (on[u]) {
+                float *o = r.out + 3 * (own[u] + base);
+                o[0] = y[u].x; o[1] = y[u].y; o[2] = y[u].z;
+            }
+}
+
+typedef void (*LLKernel)(LLRun);
+
+template <int SPT, bool LOCAL>
+LLKernel ll_kernel_z(int z)
+{
+    if (SPT <= 2 && z == 4) return ll_persistent<SPT <= 2 ? SPT : 1, 4, LOCAL>;
+    if (SPT <= 2 && z == 6) return ll_persistent<SPT <= 2 ? SPT : 1, 6, LOCAL>;
+    return ll_persistent<SPT, 0, LOCAL>;
+}
+
+// A persistent route for the run: kernel, grid, block, shared memory; kernel = null when
+// the system is too large for one.
+struct LLRoute {
+    LLKernel k = nullptr;
+    bool local = false;
+    unsigned grid = 0, block = 0;
+    size_t smem = 0;
+    bool stage_frames = false;
+};
+
+// One block per sample up to 2048 sites (two per thread; the state and any table must fit
+// shared memory).  Otherwise a cooperative launch, one block per SM, as few sites per
+// thread as cover the system.
+int ll_route(const LLArgs &a, LLRoute *out)
+{
+    *out = LLRoute();
+    int dev = 0, sms = 0, coop = 0;
+    ASD_CUDA_TRY(cudaGetDevice(&dev));
+    ASD_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    ASD_CUDA_TRY(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
+    const int64_t n = a.N * a.S;
+    LLRoute r;
+    // (int indices of the state arrays)
+    if (n > (int64_t)1 << 30) return ASD_OK;
+    const auto bonds = [&](int spt, int64_t slots) -> size_t {
+        return spt == 1 && (a.z == 4 || a.z == 6) ? 0 : (size_t)a.z * slots * 8;
+    };
+    // frames gathered in shared memory where it has room
+    const auto add_frames = [](LLRoute &r, size_t smem, int64_t slots) {
+        const size_t more = sizeof(float) * kLLFramePitch * (size_t)slots;
+        r.stage_frames = smem + more <= kLLMaxSmem;
+        r.smem = smem + (r.stage_frames ? more : 0);
+    };
+    if (a.N <= 2 * kLLThreads) {
+        const int spt = a.N <= kLLThreads ? 1 : 2;
+        const size_t smem = (size_t)48 * a.N + bonds(spt, a.N);
+        if (smem <= kLLMaxSmem) {
+            r.local = true;
+            r.k = spt == 1 ? ll_kernel_z<1, true>(a.z) : ll_kernel_z<2, true>(a.z);
+            r.grid = (unsigned)a.S;
+            r.block = (unsigned)(((a.N + spt - 1) / spt + 31) / 32 * 32);
+            add_frames(r, smem, a.N);
+            ASD_CUDA_TRY(cudaFuncSetAttribute(r.k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                              (int)r.smem));
+            *out = r;
+            return ASD_OK;
+        }
+    }
+    if (!coop) return ASD_OK;
+    for (int spt = 1; spt <= kLLMaxSpt; spt *= 2) {
+        if ((int64_t)sms * kLLThreads * spt < n) continue;
+        // spread the sites over all SMs, whole warps per block
+        const int64_t per = (n + (int64_t)sms * spt - 1) / ((int64_t)sms * spt);
+        r.block = (unsigned)((per + 31) / 32 * 32);
+        r.grid = (unsigned)((n + (int64_t)r.block * spt - 1) / ((int64_t)r.block * spt));
+        r.smem = bonds(spt, (int64_t)spt * r.block);
+        if (r.smem > kLLMaxSmem) return ASD_OK;
+        add_frames(r, r.smem, (int64_t)spt * r.block);
+        r.k = spt == 1 ? ll_kernel_z<1, false>(a.z)
+                       : spt == 2 ? ll_kernel_z<2, false>(a.z) : ll_kernel_z<4, false>(a.z);
+        ASD_CUDA_TRY(cudaFuncSetAttribute(r.k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          (int)r.smem));
+        int per_sm = 0;
+        ASD_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, r.k, (int)r.block,
+                                                                   r.smem));
+        if ((int64_t)per_sm * sms >= r.grid) *out = r;
+        return ASD_OK;
+    }
+    return ASD_OK;
+}
+
+// The whole run with the work buffers at ws (48 bytes per site-sample, 16-byte aligned) and
+// the barrier count at bar.
+int ll_run(const LLArgs &a, const LLRoute &rt, const float *spins0, float dt, int n_frames,
+           int stride, float *traj, float *spins_out, void *ws, unsigned *bar, cudaStream_t s)
+{
+    const int64_t n = a.N * a.S;
+    const int64_t steps = (int64_t)(n_frames - 1) * stride;
+    if (rt.k) {
+        LLRun r{};
+        r.a = a;
+        r.Y = static_cast<float4 *>(ws);
+        r.T1 = r.Y + n;
+        r.T2 = r.T1 + n;
+        r.bar = bar;
+        r.traj = traj;
+        r.F = n_frames;
+        r.stride = stride;
+        r.dt = dt;
+        r.stage_frames = rt.stage_frames;
+        r.err = device_error_word();
+        if (!r.err) return ASD_ECUDA;
+        const float *in = spins0;
+        int64_t st = 0;
+        do {
+            r.step0 = st;
+            r.step1 = std::min<int64_t>(steps, st + kLLStepsPerLaunch);
+            r.in = in;
+            // between launches the state goes through the first 12 bytes per site of T1
+            r.out = r.step1 == steps ? spins_out : reinterpret_cast<float *>(r.T1);
+            if (rt.local) {
+                rt.k<<<rt.grid, rt.block, rt.smem, s>>>(r);
+                ASD_CUDA_TRY(cudaGetLastError());
+            } else {
+                ASD_CUDA_TRY(cudaMemsetAsync(bar, 0, sizeof(unsigned), s));
+                void *args[] = {&r};
+                ASD_CUDA_TRY(cudaLaunchCooperativeKernel((const void *)rt.k, dim3(rt.grid),
+                                                         dim3(rt.block), args, rt.smem, s));
+            }
+            in = r.out;
+            st = r.step1;
+        } while (st < steps);
+        return ASD_OK;
+    }
+    const size_t bytes = sizeof(float) * 3 * (size_t)n;
+    // every buffer is written before it is read: Y by the copy, acc by stage 1, T1 / T2
+    // by the stage that produces them, so no clearing is needed
+    float *Y = static_cast<float *>(ws), *T1 = Y + 3 * n, *T2 = Y + 6 * n, *acc = Y + 9 * n;
+    const unsigned blocks = (unsigned)((n + 255) / 256);
+    ASD_CUDA_TRY(cudaMemcpyAsync(Y, spins0, bytes, cudaMemcpyDeviceToDevice, s));
+    write_frame0<<<blocks, 256, 0, s>>>(Y, a.N, a.S, traj, n_frames);
+    for (int f = 1; f < n_frames; ++f) {
+        for (int k = 0; k < stride; ++k) {
+            const int frame = k == stride - 1 ? f : -1;
+            rk4_stage<1><<<blocks, 256, 0, s>>>(a, Y, Y, T1, acc, dt, traj, n_frames, -1);
+            rk4_stage<2><<<blocks, 256, 0, s>>>(a, Y, T1, T2, acc, dt, traj, n_frames, -1);
+            rk4_stage<3><<<blocks, 256, 0, s>>>(a, Y, T2, T1, acc, dt, traj, n_frames, -1);
+            rk4_stage<4><<<blocks, 256, 0, s>>>(a, Y, T1, nullptr, acc, dt, traj, n_frames, frame);
+        }
+    }
+    ASD_CUDA_TRY(cudaGetLastError());
+    if (spins_out)
+        ASD_CUDA_TRY(cudaMemcpyAsync(spins_out, Y, bytes, cudaMemcpyDeviceToDevice, s));
+    return ASD_OK;
+}
+
 }  // namespace
 }  // namespace asd
 
@@ -123,39 +534,18 @@ extern "C" int asd_ll_integrate(const asd_system *sys, int n_samples, const floa
     ASD_CHECK_ARG(n_samples >= 1 && n_frames >= 1 && stride >= 1, "bad n_samples/n_frames/stride");
     cudaStream_t s = (cudaStream_t)stream;
     LLArgs a{sys->n_sites, n_samples, sys->z, sys->nbr, sys->J, sys->Hz, sys->D, sys->A};
+    LLRoute rt;
+    int rc = ll_route(a, &rt);
+    if (rc) return rc;
     const int64_t n = sys->n_sites * n_samples;
-    const size_t bytes = sizeof(float) * 3 * (size_t)n;
-    float *ws = nullptr;
-    ASD_CUDA_TRY(cudaMallocAsync(&ws, 4 * bytes, s));
-    float *Y = ws, *T1 = ws + 3 * n, *T2 = ws + 6 * n, *acc = ws + 9 * n;
-    int rc = ASD_OK;
-    const unsigned blocks = (unsigned)((n + 255) / 256);
-    do {
-        if (cudaMemcpyAsync(Y, spins0, bytes, cudaMemcpyDeviceToDevice, s) != cudaSuccess) {
-            rc = ASD_ECUDA;
-            break;
-        }
-        write_frame0<<<blocks, 256, 0, s>>>(Y, sys->n_sites, n_samples, traj, n_frames);
-        for (int f = 1; f < n_frames; ++f) {
-            for (int k = 0; k < stride; ++k) {
-                const int frame = k == stride - 1 ? f : -1;
-                rk4_stage<1><<<blocks, 256, 0, s>>>(a, Y, Y, T1, acc, dt, traj, n_frames, -1);
-                rk4_stage<2><<<blocks, 256, 0, s>>>(a, Y, T1, T2, acc, dt, traj, n_frames, -1);
-                rk4_stage<3><<<blocks, 256, 0, s>>>(a, Y, T2, T1, acc, dt, traj, n_frames, -1);
-                rk4_stage<4><<<blocks, 256, 0, s>>>(a, Y, T1, nullptr, acc, dt, traj, n_frames,
-                                                    frame);
-            }
-        }
-        if (cudaGetLastError() != cudaSuccess) {
-            rc = ASD_ECUDA;
-            break;
-        }
-        if (spins_out &&
-            cudaMemcpyAsync(spins_out, Y, bytes, cudaMemcpyDeviceToDevice, s) != cudaSuccess)
-            rc = ASD_ECUDA;
-    } while (0);
-    cudaFreeAsync(ws, s);
-    if (rc == ASD_ECUDA) set_error_text("asd_ll_integrate: launch failed");
+    char *ws = nullptr;
+    // (a block per sample in one launch keeps everything on chip)
+    const bool need = !rt.local || (int64_t)(n_frames - 1) * stride > kLLStepsPerLaunch;
+    const size_t bytes = 48 * (size_t)n;
+    if (need) ASD_CUDA_TRY(cudaMallocAsync(&ws, bytes + 16, s));
+    rc = ll_run(a, rt, spins0, dt, n_frames, stride, traj, spins_out, ws,
+                reinterpret_cast<unsigned *>(ws + bytes), s);
+    if (need) cudaFreeAsync(ws, s);
     return rc;
 }
 
@@ -172,8 +562,9 @@ namespace {
 constexpr int64_t kLLStaticMaxSiteSamples = 1 << 18;  // n_sites * n_samples limit
 constexpr int kLLStaticMaxDevices = 64;
 
-// 4 buffers x 3 components x 262144 site-samples x 4 B = 12 MiB per device
-static __device__ __align__(256) float g_ll_scratch[4 * 3 * kLLStaticMaxSiteSamples];
+// 48 B x 262144 site-samples = 12 MiB per device (three 16-byte state buffers, or four 12-byte
+// ones), then the grid barrier's count
+static __device__ __align__(256) float g_ll_scratch[4 * 3 * kLLStaticMaxSiteSamples + 64];
 
 std::mutex g_ll_scratch_mu;
 struct ScratchSlot {
@@ -254,27 +645,11 @@ extern "C" int asd_ll_integrate_noalloc(const asd_system *sys, int n_samples, co
     float *ws = nullptr;
     int rc = ll_scratch_address(&ws);
     if (rc) return rc;
-    cudaStream_t s = (cudaStream_t)stream;
     LLArgs a{sys->n_sites, n_samples, sys->z, sys->nbr, sys->J, sys->Hz, sys->D, sys->A};
-    const int64_t n = sys->n_sites * n_samples;
-    const size_t bytes = sizeof(float) * 3 * (size_t)n;
-    // every buffer is written before it is read: Y by the copy, acc by stage 1, T1 / T2
-    // by the stage that produces them, so no clearing is needed
-    float *Y = ws, *T1 = ws + 3 * n, *T2 = ws + 6 * n, *acc = ws + 9 * n;
-    const unsigned blocks = (unsigned)((n + 255) / 256);
-    ASD_CUDA_TRY(cudaMemcpyAsync(Y, spins0, bytes, cudaMemcpyDeviceToDevice, s));
-    write_frame0<<<blocks, 256, 0, s>>>(Y, sys->n_sites, n_samples, traj, n_frames);
-    for (int f = 1; f < n_frames; ++f) {
-        for (int k = 0; k < stride; ++k) {
-            const int frame = k == stride - 1 ? f : -1;
-            rk4_stage<1><<<blocks, 256, 0, s>>>(a, Y, Y, T1, acc, dt, traj, n_frames, -1);
-            rk4_stage<2><<<blocks, 256, 0, s>>>(a, Y, T1, T2, acc, dt, traj, n_frames, -1);
-            rk4_stage<3><<<blocks, 256, 0, s>>>(a, Y, T2, T1, acc, dt, traj, n_frames, -1);
-            rk4_stage<4><<<blocks, 256, 0, s>>>(a, Y, T1, nullptr, acc, dt, traj, n_frames, frame);
-        }
-    }
-    ASD_CUDA_TRY(cudaGetLastError());
-    if (spins_out)
-        ASD_CUDA_TRY(cudaMemcpyAsync(spins_out, Y, bytes, cudaMemcpyDeviceToDevice, s));
-    return ASD_OK;
+    LLRoute rt;
+    rc = ll_route(a, &rt);
+    if (rc) return rc;
+    return ll_run(a, rt, spins0, dt, n_frames, stride, traj, spins_out, ws,
+                  reinterpret_cast<unsigned *>(ws + 4 * 3 * kLLStaticMaxSiteSamples),
+                  (cudaStream_t)stream);
 }
