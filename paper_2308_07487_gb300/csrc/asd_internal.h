@@ -43,7 +43,7 @@ enum DeviceError : int {
     DEV_TIMEOUT_MMA = 2,
     DEV_TIMEOUT_EPI = 3,
     DEV_TIMEOUT_SELFTEST = 4,
-    DEV_TIMEOUT_LL = 5,
+    DEV_TIMEOUT_GRID = 5,
     DEV_BOUNDS = 256
 };
 int *device_error_word();          // device address of the word for the current device

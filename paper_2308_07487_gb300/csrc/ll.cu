@@ -21,6 +21,7 @@
 #include <algorithm>
 
 #include "asd_internal.h"
+#include "grid_barrier.cuh"
 
 namespace asd {
 namespace {
@@ -128,7 +129,6 @@ constexpr int kLLThreads = 1024;
 constexpr int kLLMaxSpt = 4;                       // sites per thread
 constexpr size_t kLLMaxSmem = 220 * 1024;
 constexpr int kLLStepsPerLaunch = 4096;            // other streams' work gets in between
-constexpr unsigned long long kLLTimeoutNs = 4000000000ull;
 
 struct LLRun {
     LLArgs a;
@@ -146,38 +146,6 @@ struct LLRun {
 };
 constexpr int kLLFrames = 4;
 constexpr int kLLFramePitch = 3 * kLLFrames + 1;   // words per site (odd: no bank conflicts)
-
-// Barrier over all blocks of a cooperative launch: the count reaches `target` once every
-// block has arrived.  The release before the arrival and the acquire after the wait order
-// all blocks' global stores and loads around it (the acquire also drops this SM's L1 lines).
-// Bounded: false for every thread of the block after kLLTimeoutNs.
-__device__ __forceinline__ bool grid_barrier(unsigned *bar, unsigned target, int *err)
-{
-    __syncthreads();
-    int ok = 1;
-    if (threadIdx.x == 0) {
-        __threadfence();
-        asm volatile("red.relaxed.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
-        unsigned long long t0 = 0;
-        for (unsigned it = 0;; ++it) {
-            unsigned v;
-            asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
-            if ((int)(v - target) >= 0) break;
-            if ((it & 1023u) == 1023u) {
-                unsigned long long now;
-                asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
-                if (t0 == 0) t0 = now;
-                else if (now - t0 > kLLTimeoutNs) {
-                    atomicCAS(err, 0, (int)DEV_TIMEOUT_LL);
-                    ok = 0;
-                    break;
-                }
-            }
-        }
-        __threadfence();
-    }
-    return __syncthreads_and(ok) != 0;
-}
 
 // All steps of a launch.  Bound by the latency of a stage (380 to 640 dependent stages, each
 // a few hundred cycles of loads and arithmetic), not by bandwidth, so the work is to take the
