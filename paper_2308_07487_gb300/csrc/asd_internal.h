@@ -135,7 +135,7 @@ struct EpiParams {
     int npass;              // passes of kPhaseQ q-vectors (0 without phase weights)
     int q_parts;            // 1: cosine part of the phase sum; 2: cosine and sine parts
     const float2 *cs;       // [N][nq_pad] (cos, sin)(q.r_i)
-    const float2 *csT;      // the same by q: [nq_pad][cs_ld] (tensor forms)
+    const float2 *csT;      // the same by q: [nq_pad][cs_ld], zero past the last site
     int64_t cs_ld;          // row length of csT
     double *C_sum;          // [n_t][n_bins]
     double *Sq_sum;         // [n_t][n_q]
@@ -230,7 +230,9 @@ struct asd_corr_plan {
     size_t ws_bytes;
     void *A[2][asd::kMaxCopies];
     void *B[2];
-    float *Bf32;               // FP32 form: B operand
+    float *Af32;              // FP32 form: A operand by K, every value twice [R][ld32]
+    float *Bf32;               // FP32 form: B operand by K [Kb][ld32]
+    int64_t ld32;              // sites rounded up to whole tiles
     float *meanB;              // [N][3] centring means
     // geometry (device)
     int4 *coords;
@@ -240,7 +242,7 @@ struct asd_corr_plan {
     int no_drop, pos_ok;       // see EpiParams
     uint16_t *lut;             // lattice d2 -> bin table (nullptr when d2 can reach kLutMax)
     int n_lut;
-    float2 *cs, *csT;          // (cos, sin)(q.r_i) by site; by q (tensor forms)
+    float2 *cs, *csT;          // (cos, sin)(q.r_i) by site; by q [nq_pad][ld32]
     void *W;                   // phase column weights [2 planes][npass * 128][Wld] BF16
     int64_t Wld;               // row length of W (N rounded up to 8)
     double *sqF;               // separable phase form: transforms [2 n_q][S*3F] (n_q > 0)
@@ -279,8 +281,8 @@ int launch_prep(asd_corr_plan *p, const float *traj, int64_t row_begin, int64_t 
                 cudaStream_t s);
 int launch_counts(asd_corr_plan *p, cudaStream_t s, unsigned long long *d_counts);
 // pc_simt.cu
-int launch_simt(asd_corr_plan *p, const float *traj, int64_t row_begin, int64_t row_end,
-                int t_begin, int t_end, double *C_sum, double *Sq_sum, cudaStream_t s);
+int launch_simt(asd_corr_plan *p, int64_t row_begin, int64_t row_end, int t_begin, int t_end,
+                double *C_sum, double *Sq_sum, cudaStream_t s);
 // pc_tc.cu
 int tc_configure(asd_corr_plan *p);    // stages / smem for the plan's form
 int launch_tc(const TcProblem *d_probs, int n_probs, const TcDims &one, int64_t total_tiles,

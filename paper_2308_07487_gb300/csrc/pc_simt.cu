@@ -9,20 +9,31 @@
 // through cos(a-b) = cos a cos b + sin a sin b with warp shuffles (Section 3.3, the
 // shuffle + shared-memory + atomic reduction), then one FP64 global atomic per bin
 // (and per q) per tile.  In the deterministic mode the same sums are 64-bit fixed point
-// (integer atomics, the same bits in any order).  A is read straight from the trajectory row at the K-offset
-// s*3F + 3t; B is the prepared, zero-padded FP32 copy.
+// (integer atomics, the same bits in any order).
+//
+// Operands are prepared by K: A[k][site] of the whole trajectory row (the displacement's K
+// window is a row offset, so no shifted copies) and B[k][site], zero padded.  Both go to shared
+// memory as they are (cp.async, no registers, a three-stage pipeline of 16 k).  A thread's
+// 8 x 8 outputs are 8 x 4 pairs of columns under packed FMAs: 32 instead of 64 issue slots
+// per k, with which the FP32 pipes, which bound the kernel, stay 75 % busy.  Measured on the
+// 24^3 glass, K = 1536, 96 bins and 32 q, 2 displacements: 37.8 -> 22.1 ms (31 -> 53 TFLOP/s;
+// bins only 58, K = 6144 bins only 60); the steps: operands by K with cp.async and packed FMAs
+// 28.1 (scalar FMAs 29.4; A stored twice per value to save packing 31.6), weights by q in the
+// phase sums (whole lines instead of 16 per load) 24.6, 16 k per stage instead of 8 22.1.
 #include "asd_internal.h"
 #include "geom.cuh"
 
 namespace asd {
 namespace {
 
-constexpr int TM = 128, TN = 128, TK = 8;
+constexpr int TM = 128, TN = 128, TK = 16;
+constexpr int kStages = 3;
+constexpr int kStageFloats = TK * (TM + TN);   // A twice, B
 
 struct SimtParams {
-    const float *traj;
-    const float *B;
-    int64_t R;        // trajectory row length S*3F
+    const float *A;  // [R][ld], every value twice
+    const float *B;   // [S*Kseg][ld]
+    int64_t ld;       // sites, padded to whole tiles
     int F3;
     int K3;           // 3*T0
     int Kseg;         // B segment per sample
@@ -30,17 +41,35 @@ struct SimtParams {
     int N;
     int row_begin, row_end;
     int t_begin;      // displacement of grid slice blockIdx.z = 0
+    int a16;          // A rows start on 16 bytes (an even first row)
     int warp_bins;    // per-warp FP32 bin copies after the FP64 arrays
     EpiParams e;
     int *err;         // device error word (index checks of a checked build)
 };
 
-// (two CTAs per SM: at most 128 registers a thread)
-__global__ void __launch_bounds__(256, 2) simt_kernel(SimtParams P)
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, uint32_t bytes)
 {
-    __shared__ __align__(16) float As[2][TK][TM];
-    __shared__ __align__(16) float Bs[2][TK][TN];
-    extern __shared__ double red[];  // [n_bins] then [n_q][q_parts], then [8][n_bins] FP32
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes)
+                 : "memory");
+}
+__device__ __forceinline__ void cp_async4(uint32_t dst, const void *src, uint32_t bytes)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(bytes)
+                 : "memory");
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c)
+{
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+
+// (two CTAs per SM: at most 128 registers a thread)
+__global__ void __launch_bounds__(256, 2) simt_kernel(const __grid_constant__ SimtParams P)
+{
+    // pipeline stages, then [n_bins] and [n_q][q_parts] FP64, then [8][n_bins] FP32
+    extern __shared__ __align__(16) float dyn[];
+    double *red = reinterpret_cast<double *>(dyn + kStages * kStageFloats);
     double *sbins = red;
     double *sq = red + P.e.n_bins;
     float *wbins = reinterpret_cast<float *>(sq + P.e.n_q * P.e.q_parts);
@@ -59,66 +88,84 @@ __global__ void __launch_bounds__(256, 2) simt_kernel(SimtParams P)
     if (wb_on)
         for (int k = tid; k < 8 * P.e.n_bins; k += 256) wbins[k] = 0.f;
 
-    // loader mapping: one row (or column) and 4 consecutive k per thread
-    const int lr = tid >> 1, lk = (tid & 1) * 4;
-    const int li = m0 + lr, lj = n0 + lr;
-    const bool a_ok = li < P.row_end;
-    const bool b_ok = lj < P.N;
-    const float *arow = P.traj + (int64_t)(a_ok ? li : 0) * P.R + 3 * t;
-    const float *brow = P.B + (int64_t)(b_ok ? lj : 0) * P.S * P.Kseg;
-
     const int steps_per_seg = P.Kseg / TK;
     const int n_steps = P.S * steps_per_seg;
-    float ra[4], rb[4];
+    // a stage: 8 k of 128 sites, A as float2 (512 16-byte words: two per thread), B 256.
+    // Rows past the range and k past 3*T0 read as zeros.
+    int ls = 0, lk = 0;   // sample and k of the next stage to load
     auto load = [&](int st) {
-        const int s = st / steps_per_seg;
-        const int kl = (st % steps_per_seg) * TK + lk;
-        const float *ap = arow + (int64_t)s * P.F3 + kl;
+        if (st < n_steps) {
+            float *buf = dyn + (st % kStages) * kStageFloats;
+            const uint32_t da = (uint32_t)__cvta_generic_to_shared(buf);
+            const float *A = P.A + ((int64_t)ls * P.F3 + 3 * t + lk) * P.ld + m0;
 #pragma unroll
-        for (int u = 0; u < 4; ++u) ra[u] = (a_ok && kl + u < P.K3) ? __ldg(ap + u) : 0.f;
-        float4 bv = b_ok ? __ldg(reinterpret_cast<const float4 *>(brow + (int64_t)s * P.Kseg + kl))
-                         : make_float4(0.f, 0.f, 0.f, 0.f);
-        rb[0] = bv.x; rb[1] = bv.y; rb[2] = bv.z; rb[3] = bv.w;
-    };
-    auto store = [&](int buf) {
+            for (int u = 0; u < TK / 8; ++u) {
+                const int e = tid + 256 * u, k = e >> 5, r = (e & 31) * 4;   // four sites
+                const int left = lk + k < P.K3 ? min(4, max(0, P.row_end - m0 - r)) : 0;
+                const float *src = left ? A + k * P.ld + r : P.A;
+                const uint32_t dst = da + (uint32_t)(k * TM + r) * 4;
+                if (P.a16) {
+                    cp_async16(dst, src, 4u * left);
+                } else {
+                    for (int q = 0; q < 4; ++q) cp_async4(dst + 4 * q, left > q ? src + q : P.A, left > q ? 4u : 0u);
+                }
+            }
+            const float *B = P.B + ((int64_t)ls * P.Kseg + lk) * P.ld + n0;
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            As[buf][lk + u][lr] = ra[u];
-            Bs[buf][lk + u][lr] = rb[u];
+            for (int u = 0; u < TK / 8; ++u) {
+                const int e = tid + 256 * u, k = e >> 5, c = (e & 31) * 4;
+                cp_async16(da + (uint32_t)(TK * TM + k * TN + c) * 4, B + k * P.ld + c, 16u);
+            }
+            lk += TK;
+            if (lk == P.Kseg) {
+                lk = 0;
+                ++ls;
+            }
         }
+        asm volatile("cp.async.commit_group;" ::: "memory");
     };
 
+    uint64_t acc2[8][4];
+#pragma unroll
+    for (int r = 0; r < 8; ++r)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) acc2[r][c] = 0ull;
+
+    for (int st = 0; st < kStages - 1; ++st) load(st);
+    for (int st = 0; st < n_steps; ++st) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(kStages - 2) : "memory");
+        __syncthreads();   // the stage is in, and every thread is done with the one before
+        load(st + kStages - 1);
+        const float *As = dyn + (st % kStages) * kStageFloats;
+        const float *Bs = As + TK * TM;
+#pragma unroll
+        for (int kk = 0; kk < TK; ++kk) {
+            uint64_t a[8], b[4];
+            const float4 *ap = reinterpret_cast<const float4 *>(As + kk * TM) + ty;
+            const ulonglong2 *bp = reinterpret_cast<const ulonglong2 *>(Bs + kk * TN) + tx;
+            ulonglong2 v;
+            float4 f = ap[0], h = ap[16];
+#define DUP(d, s) asm("mov.b64 %0, {%1, %1};" : "=l"(d) : "f"(s))
+            DUP(a[0], f.x); DUP(a[1], f.y); DUP(a[2], f.z); DUP(a[3], f.w);
+            DUP(a[4], h.x); DUP(a[5], h.y); DUP(a[6], h.z); DUP(a[7], h.w);
+            v = bp[0];  b[0] = v.x; b[1] = v.y;
+            v = bp[16]; b[2] = v.x; b[3] = v.y;
+#pragma unroll
+            for (int r = 0; r < 8; ++r)
+#pragma unroll
+                for (int c = 0; c < 4; ++c) acc2[r][c] = fma2(a[r], b[c], acc2[r][c]);
+        }
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
     float acc[8][8];
 #pragma unroll
     for (int r = 0; r < 8; ++r)
 #pragma unroll
-        for (int c = 0; c < 8; ++c) acc[r][c] = 0.f;
-
-    load(0);
-    store(0);
-    __syncthreads();
-    for (int st = 0; st < n_steps; ++st) {
-        const int buf = st & 1;
-        if (st + 1 < n_steps) load(st + 1);
-#pragma unroll
-        for (int kk = 0; kk < TK; ++kk) {
-            float a[8], b[8];
-            float4 a0 = *reinterpret_cast<const float4 *>(&As[buf][kk][ty * 4]);
-            float4 a1 = *reinterpret_cast<const float4 *>(&As[buf][kk][64 + ty * 4]);
-            float4 b0 = *reinterpret_cast<const float4 *>(&Bs[buf][kk][tx * 4]);
-            float4 b1 = *reinterpret_cast<const float4 *>(&Bs[buf][kk][64 + tx * 4]);
-            a[0] = a0.x; a[1] = a0.y; a[2] = a0.z; a[3] = a0.w;
-            a[4] = a1.x; a[5] = a1.y; a[6] = a1.z; a[7] = a1.w;
-            b[0] = b0.x; b[1] = b0.y; b[2] = b0.z; b[3] = b0.w;
-            b[4] = b1.x; b[5] = b1.y; b[6] = b1.z; b[7] = b1.w;
-#pragma unroll
-            for (int r = 0; r < 8; ++r)
-#pragma unroll
-                for (int c = 0; c < 8; ++c) acc[r][c] = fmaf(a[r], b[c], acc[r][c]);
-        }
-        if (st + 1 < n_steps) store(buf ^ 1);
-        __syncthreads();
-    }
+        for (int c = 0; c < 4; ++c)
+            asm("mov.b64 {%0, %1}, %2;"
+                : "=f"(acc[r][2 * c]), "=f"(acc[r][2 * c + 1])
+                : "l"(acc2[r][c]));
 
     // ---------------- epilogue: reduce the tile ----------------
     int ri[8], cj[8];
@@ -157,13 +204,16 @@ __global__ void __launch_bounds__(256, 2) simt_kernel(SimtParams P)
         for (int q = 0; q < e.n_q; ++q) {
             float part = 0.f, part_s = 0.f;
             float2 wc[8];
+            const float2 *csq = e.csT + (int64_t)q * e.cs_ld;   // a row per q: whole lines
 #pragma unroll
-            for (int c = 0; c < 8; ++c)
-                wc[c] = cj[c] < P.N ? e.cs[(int64_t)cj[c] * e.nq_pad + q] : make_float2(0.f, 0.f);
+            for (int c = 0; c < 8; c += 2) {   // two sites per 16-byte load (zeros past N)
+                const float4 w = __ldg(reinterpret_cast<const float4 *>(csq + cj[c]));
+                wc[c] = make_float2(w.x, w.y);
+                wc[c + 1] = make_float2(w.z, w.w);
+            }
 #pragma unroll
             for (int r = 0; r < 8; ++r) {
-                const float2 wr = ri[r] < P.row_end ? e.cs[(int64_t)ri[r] * e.nq_pad + q]
-                                                    : make_float2(0.f, 0.f);
+                const float2 wr = ri[r] < P.row_end ? __ldg(csq + ri[r]) : make_float2(0.f, 0.f);
                 float u = 0.f, v = 0.f;
 #pragma unroll
                 for (int c = 0; c < 8; ++c) {
@@ -171,7 +221,7 @@ __global__ void __launch_bounds__(256, 2) simt_kernel(SimtParams P)
                     v = fmaf(wc[c].y, acc[r][c], v);
                 }
                 part = fmaf(wr.x, u, fmaf(wr.y, v, part));        // cos(a - b)
-                part_s = fmaf(wr.y, u, fmaf(-wr.x, v, part_s));   // sin(a - b)
+                if (e.q_parts == 2) part_s = fmaf(wr.y, u, fmaf(-wr.x, v, part_s));  // sin(a - b)
             }
             // the warp's 32 partial sums (64 pairs each) in FP32, one FP64 add per warp
             // (FP64 arithmetic runs on a narrow pipe on this part)
@@ -211,13 +261,14 @@ __global__ void __launch_bounds__(256, 2) simt_kernel(SimtParams P)
 
 }  // namespace
 
-int launch_simt(asd_corr_plan *p, const float *traj, int64_t row_begin, int64_t row_end,
-                int t_begin, int t_end, double *C_sum, double *Sq_sum, cudaStream_t s)
+int launch_simt(asd_corr_plan *p, int64_t row_begin, int64_t row_end, int t_begin, int t_end,
+                double *C_sum, double *Sq_sum, cudaStream_t s)
 {
     SimtParams P{};
-    P.traj = traj;
+    P.A = p->Af32;
     P.B = p->Bf32;
-    P.R = p->R;
+    P.ld = p->ld32;
+    P.a16 = (row_begin & 3) == 0;
     P.F3 = 3 * p->F;
     P.K3 = 3 * p->T0;
     P.Kseg = (int)p->Kseg;
@@ -240,7 +291,8 @@ int launch_simt(asd_corr_plan *p, const float *traj, int64_t row_begin, int64_t 
     e.thr = p->thr;
     e.nq_pad = (p->n_q + kQChunk - 1) / kQChunk * kQChunk;
     e.q_parts = p->q_parts;
-    e.cs = p->cs;
+    e.csT = p->csT;
+    e.cs_ld = p->ld32;
     e.C_sum = C_sum;
     e.Sq_sum = Sq_sum;
     e.C_fix = p->C_fix;
@@ -255,9 +307,12 @@ int launch_simt(asd_corr_plan *p, const float *traj, int64_t row_begin, int64_t 
         return ASD_EUNSUPPORTED;
     }
     size_t smem = sizeof(double) * (p->n_bins + p->n_q * p->q_parts);
-    // per-warp FP32 bin copies where they fit the default 48 KB of dynamic shared memory
+    // per-warp FP32 bin copies where they and the FP64 sums fit 48 KB
     P.warp_bins = !p->d.deterministic && smem + sizeof(float) * 8 * p->n_bins <= 48 * 1024;
     if (P.warp_bins) smem += sizeof(float) * 8 * p->n_bins;
+    smem += sizeof(float) * kStages * kStageFloats;
+    ASD_CUDA_TRY(cudaFuncSetAttribute(simt_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)smem));
     simt_kernel<<<grid, 256, smem, s>>>(P);
     ASD_CUDA_TRY(cudaGetLastError());
     return ASD_OK;

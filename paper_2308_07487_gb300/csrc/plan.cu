@@ -148,7 +148,7 @@ static EpiParams epi_of(const asd_corr_plan *p)
     e.q_parts = p->q_parts;
     e.cs = p->cs;
     e.csT = p->csT;
-    e.cs_ld = p->N;
+    e.cs_ld = p->ld32;
     e.C_fix = p->C_fix;
     e.Sq_fix = p->Sq_fix;
     e.fix_scale = p->d.deterministic ? p->fix_scale : nullptr;
@@ -600,12 +600,15 @@ int asd_pair_corr_plan_create(const asd_corr_desc *d, asd_corr_plan **out)
 
     // ---- workspace ----
     size_t bytes = 0;
-    const size_t a_bytes = tc ? (size_t)p->N * p->Rpad * p->elem_bytes : 0;
-    const size_t b_bytes = (size_t)p->N * p->Kb * (tc ? p->elem_bytes : 4);
+    p->ld32 = (p->N + 127) / 128 * 128;
+    const size_t a_bytes =
+        tc ? (size_t)p->N * p->Rpad * p->elem_bytes : (size_t)p->ld32 * R * sizeof(float);
+    const size_t b_bytes = tc ? (size_t)p->N * p->Kb * p->elem_bytes
+                              : (size_t)p->ld32 * p->Kb * sizeof(float);
     const size_t r256 = 256;
     auto up = [&](size_t b) { return (b + r256 - 1) / r256 * r256; };
     if (tc) bytes += p->n_planes * p->n_copies * up(a_bytes) + p->n_planes * up(b_bytes);
-    else bytes += up(b_bytes);
+    else bytes += up(a_bytes) + up(b_bytes);
     bytes += up((size_t)p->N * 3 * sizeof(float));  // centring means
     if (cudaMalloc(&p->ws, bytes) != cudaSuccess) {
         cudaGetLastError();
@@ -620,8 +623,10 @@ int asd_pair_corr_plan_create(const asd_corr_desc *d, asd_corr_plan **out)
                 for (int c = 0; c < p->n_copies; ++c) carve(cur, a_bytes, &p->A[pl][c]);
             for (int pl = 0; pl < p->n_planes; ++pl) carve(cur, b_bytes, &p->B[pl]);
         } else {
-            void *b = nullptr;
+            void *a = nullptr, *b = nullptr;
+            carve(cur, a_bytes, &a);
             carve(cur, b_bytes, &b);
+            p->Af32 = static_cast<float *>(a);
             p->Bf32 = static_cast<float *>(b);
         }
         void *m = nullptr;
@@ -706,6 +711,18 @@ int asd_pair_corr_plan_create(const asd_corr_desc *d, asd_corr_plan **out)
             }
             if (cudaMemcpy(p->cs, cs.data(), sizeof(float2) * cs.size(), cudaMemcpyHostToDevice))
                 return fail(ASD_ECUDA);
+            // the same by q, sites padded to whole tiles
+            std::vector<float2> csT((size_t)nqp * p->ld32, make_float2(0.f, 0.f));
+            for (int64_t i = 0; i < p->N; ++i)
+                for (int q = 0; q < p->n_q; ++q)
+                    csT[(size_t)q * p->ld32 + i] = cs[(size_t)i * nqp + q];
+            if (cudaMalloc(&p->csT, sizeof(float2) * csT.size()) != cudaSuccess) {
+                cudaGetLastError();
+                return fail(ASD_ENOMEM);
+            }
+            if (cudaMemcpy(p->csT, csT.data(), sizeof(float2) * csT.size(),
+                           cudaMemcpyHostToDevice))
+                return fail(ASD_ECUDA);
             // column weights of the tensor-core phase product, pass by pass: row
             // pp * 128 + o holds cos(q.r_c) of q = 64 pp + o (o < 64) or sin(q.r_c) of
             // q = 64 pp + o - 64, zero for q >= n_q, as BF16 hi = RN(x) and
@@ -715,11 +732,9 @@ int asd_pair_corr_plan_create(const asd_corr_desc *d, asd_corr_plan **out)
                 p->Wld = (p->N + 7) / 8 * 8;
                 const size_t rows = (size_t)npass * 2 * kPhaseQ, plane = rows * p->Wld;
                 std::vector<uint16_t> W(2 * plane, 0);
-                std::vector<float2> csT((size_t)nqp * p->N, make_float2(0.f, 0.f));
                 for (int64_t c = 0; c < p->N; ++c) {
                     for (int q = 0; q < p->n_q; ++q) {
                         const double *x2 = &xs[2 * ((size_t)c * p->n_q + q)];
-                        csT[(size_t)q * p->N + c] = cs[(size_t)c * nqp + q];
                         for (int part = 0; part < 2; ++part) {
                             const size_t row = (size_t)(q / kPhaseQ) * 2 * kPhaseQ +
                                                part * kPhaseQ + q % kPhaseQ;
@@ -730,13 +745,6 @@ int asd_pair_corr_plan_create(const asd_corr_desc *d, asd_corr_plan **out)
                         }
                     }
                 }
-                if (cudaMalloc(&p->csT, sizeof(float2) * csT.size()) != cudaSuccess) {
-                    cudaGetLastError();
-                    return fail(ASD_ENOMEM);
-                }
-                if (cudaMemcpy(p->csT, csT.data(), sizeof(float2) * csT.size(),
-                               cudaMemcpyHostToDevice))
-                    return fail(ASD_ECUDA);
                 if (cudaMalloc(&p->W, sizeof(uint16_t) * W.size()) != cudaSuccess) {
                     cudaGetLastError();
                     return fail(ASD_ENOMEM);
@@ -874,7 +882,7 @@ int asd_pair_corr_contract_range(asd_corr_plan *p, int64_t row_begin, int64_t ro
     int rc = fix_begin(p, row_end - row_begin, t_begin, t_end, s);
     if (rc) return rc;
     if (!p->tc) {
-        rc = launch_simt(p, p->prepared_traj, row_begin, row_end, t_begin, t_end, C_sum, Sq_sum, s);
+        rc = launch_simt(p, row_begin, row_end, t_begin, t_end, C_sum, Sq_sum, s);
         return rc ? rc : fix_end(p, t_begin, t_end, C_sum, Sq_sum, s);
     }
     TcOverride ov{};

@@ -15,7 +15,7 @@
 // are reached with B alone.
 //
 // Precision forms: BF16 hi = RN(x); split-BF16 lo = RN(x - hi); TF32 = RNA to 10-bit
-// mantissa (the tensor core would otherwise truncate); FP32 keeps B in FP32.
+// mantissa (the tensor core would otherwise truncate); FP32: both operands by K (prep32_kernel).
 #include <cuda_bf16.h>
 
 #include "asd_internal.h"
@@ -80,10 +80,9 @@ __device__ __forceinline__ void prep_b(const float *__restrict__ traj, int64_t N
             v[u] = x;
         }
         const int64_t off = j * (int64_t)S * Kseg + kk;
-        if (FORM == ASD_FP32 || FORM == ASD_TF32) {
+        if (FORM == ASD_TF32) {
             float4 *o = reinterpret_cast<float4 *>(static_cast<float *>(out0) + off);
-            if (FORM == ASD_TF32)
-                for (int u = 0; u < 8; ++u) v[u] = tf32_round(v[u]);
+            for (int u = 0; u < 8; ++u) v[u] = tf32_round(v[u]);
             o[0] = make_float4(v[0], v[1], v[2], v[3]);
             o[1] = make_float4(v[4], v[5], v[6], v[7]);
         } else {
@@ -150,6 +149,62 @@ __device__ __forceinline__ void prep_a(const float *__restrict__ traj, int64_t r
     }
 }
 
+// FP32 form: operands by K.  32 x 32 tiles through shared memory, k along a trajectory row in,
+// sites out: A[k][i] for rows [row_begin, row_end) and every k of the row, and
+// B[s*Kseg + kl][j] = x (centred), zero for kl >= 3*T0 and for the padding sites.
+struct Prep32Args {
+    const float *traj;
+    int64_t N, ld, R, row_begin, row_end;
+    int S, F3, K3, Kseg;
+    const float *mean;
+    int center;
+    float *A;
+    float *B;
+    int64_t tiles_a_k, tiles_a, tiles_b_k, tiles;   // along k, A in all; B along k; in all
+};
+
+__global__ void __launch_bounds__(256) prep32_kernel(const __grid_constant__ Prep32Args a)
+{
+    __shared__ float tile[32][33];
+    const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
+    for (int64_t blk = blockIdx.x; blk < a.tiles; blk += gridDim.x) {
+        const bool is_a = blk < a.tiles_a;
+        const int64_t b = is_a ? blk : blk - a.tiles_a;
+        const int64_t tk = is_a ? a.tiles_a_k : a.tiles_b_k;
+        const int64_t k0 = b % tk * 32, i0 = (is_a ? a.row_begin : 0) + b / tk * 32;
+        const int64_t i1 = is_a ? a.row_end : a.N;
+#pragma unroll
+        for (int u = 0; u < 32; u += 8) {
+            const int64_t i = i0 + y + u, k = k0 + x;
+            float v = 0.f;
+            if (i < i1) {
+                if (is_a) {
+                    if (k < a.R) v = __ldg(a.traj + i * a.R + k);
+                } else {
+                    const int s = (int)(k / a.Kseg), kl = (int)(k - (int64_t)s * a.Kseg);
+                    if (s < a.S && kl < a.K3) {
+                        v = __ldg(a.traj + i * a.R + (int64_t)s * a.F3 + kl);
+                        if (a.center) v -= a.mean[3 * i + kl % 3];
+                    }
+                }
+            }
+            tile[y + u][x] = v;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < 32; u += 8) {
+            const int64_t k = k0 + y + u, i = i0 + x;
+            const float v = tile[x][y + u];
+            if (is_a) {
+                if (k < a.R && i < i1) a.A[k * a.ld + i] = v;
+            } else if (k < (int64_t)a.S * a.Kseg && i < a.ld) {
+                a.B[k * a.ld + i] = v;
+            }
+        }
+        __syncthreads();
+    }
+}
+
 // Both operands in one launch, the first blocks_b blocks the B operand and the rest the A
 // copies (a launch costs a call of a small problem 2 us, as much as its preparation:
 // 16 x 16 sites, T0 = 64, preparation to normalisation 33.1 -> 30.8 us).
@@ -171,7 +226,7 @@ __global__ void __launch_bounds__(256) prep_kernel(const __grid_constant__ PrepA
     if (blockIdx.x < a.blocks_b)
         prep_b<FORM>(a.traj, a.N, a.S, a.F, a.T0, a.Kseg, a.mean, a.center, a.b0, a.b1,
                      blockIdx.x, a.blocks_b);
-    else if constexpr (FORM != ASD_FP32)
+    else
         prep_a<FORM>(a.traj, a.row_begin, a.row_end, a.R, a.Rpad, a.cp,
                      blockIdx.x - a.blocks_b, gridDim.x - a.blocks_b);
 }
@@ -193,6 +248,31 @@ int launch_prep(asd_corr_plan *p, const float *traj, int64_t row_begin, int64_t 
         means_kernel<<<(unsigned)((p->N + 7) / 8), 256, 0, s>>>(traj, p->N, S, F, T0, p->meanB);
         ASD_CUDA_TRY(cudaGetLastError());
     }
+    if (!p->tc) {
+        Prep32Args a{};
+        a.traj = traj;
+        a.N = p->N;
+        a.ld = p->ld32;
+        a.R = p->R;
+        a.row_begin = row_begin;
+        a.row_end = row_end;
+        a.S = S;
+        a.F3 = 3 * F;
+        a.K3 = 3 * T0;
+        a.Kseg = (int)p->Kseg;
+        a.mean = p->meanB;
+        a.center = p->center;
+        a.A = p->Af32;
+        a.B = p->Bf32;
+        a.tiles_a_k = (p->R + 31) / 32;
+        a.tiles_a = a.tiles_a_k * ((row_end - row_begin + 31) / 32);
+        a.tiles_b_k = (p->Kb + 31) / 32;
+        a.tiles = a.tiles_a + a.tiles_b_k * (p->ld32 / 32);
+        const int64_t blocks = a.tiles < (1 << 20) ? a.tiles : 1 << 20;
+        prep32_kernel<<<(unsigned)blocks, 256, 0, s>>>(a);
+        ASD_CUDA_TRY(cudaGetLastError());
+        return ASD_OK;
+    }
     PrepArgs a{};
     a.traj = traj;
     a.N = p->N;
@@ -202,7 +282,7 @@ int launch_prep(asd_corr_plan *p, const float *traj, int64_t row_begin, int64_t 
     a.Kseg = (int)p->Kseg;
     a.mean = p->meanB;
     a.center = p->center;
-    a.b0 = p->tc ? p->B[0] : p->Bf32;
+    a.b0 = p->B[0];
     a.b1 = p->B[1];
     a.blocks_b = grid_for(p->N * p->Kb / 8, p->sm_count);
     a.row_begin = row_begin;
@@ -212,11 +292,10 @@ int launch_prep(asd_corr_plan *p, const float *traj, int64_t row_begin, int64_t 
     for (int pl = 0; pl < p->n_planes; ++pl)
         for (int c = 0; c < p->n_copies; ++c) a.cp.p[pl][c] = p->A[pl][c];
     unsigned blocks = a.blocks_b;
-    if (p->tc && row_end > row_begin)
+    if (row_end > row_begin)
         blocks += grid_for((row_end - row_begin) * (p->Rpad / (p->prec == ASD_TF32 ? 4 : 8)),
                            p->sm_count);
     switch (p->prec) {
-    case ASD_FP32: prep_kernel<ASD_FP32><<<blocks, 256, 0, s>>>(a); break;
     case ASD_TF32: prep_kernel<ASD_TF32><<<blocks, 256, 0, s>>>(a); break;
     case ASD_BF16: prep_kernel<ASD_BF16><<<blocks, 256, 0, s>>>(a); break;
     default: prep_kernel<ASD_SPLIT_BF16><<<blocks, 256, 0, s>>>(a); break;
