@@ -3,7 +3,10 @@
 //   S(q, w_k) = dt * ( v_0 S(q, 0) + 2 sum_{t=1}^{n_t-1} v_t S(q, t) cos(w_k t dt) ),
 // with v_t = 1 (no window), 0.5 (1 + cos(pi t / n_t)) (Hann) or exp(-(t / (width n_t))^2 / 2)
 // (Gaussian).  The cosine advances by a rotation per step, re-seeded from sincos every 32
-// steps, in FP64.
+// steps, in FP64; a block (one frequency) makes its cosines once, a thread per run of 32, for
+// all q-vectors.  The FP64 pipe bounds this kernel: two operations per (frequency, q,
+// displacement) instead of six with a rotation in every thread (256 frequencies, 64 q, 128
+// displacements: 65 -> 32 us).
 #include <cuda_runtime.h>
 
 #include "asd_internal.h"
@@ -11,13 +14,16 @@
 namespace asd {
 namespace {
 
-constexpr int kMaxNt = 6000;  // window weights in shared memory (48 KB)
+constexpr int kMaxNt = 6000;  // window weights and cosines in shared memory (96 KB)
 
 __global__ void sq_omega_kernel(const double *__restrict__ S, int n_t, int n_q, double dt,
                                 int window, double width, const double *__restrict__ omega,
                                 double *__restrict__ Sqw)
 {
-    extern __shared__ double v[];
+    extern __shared__ double v[];   // [n_t] window, then [n_t] cosines
+    double *ct = v + n_t;
+    const int k = blockIdx.x;
+    const double th = omega[k] * dt;
     for (int t = threadIdx.x; t < n_t; t += blockDim.x) {
         double w = 1.0;
         if (window == 1) w = 0.5 * (1.0 + cospi((double)t / n_t));
@@ -27,23 +33,23 @@ __global__ void sq_omega_kernel(const double *__restrict__ S, int n_t, int n_q, 
         }
         v[t] = w;
     }
-    __syncthreads();
-    const int k = blockIdx.x;
-    const double th = omega[k] * dt;
     double sr, cr;
     sincos(th, &sr, &cr);  // rotation by one step
-    for (int q = threadIdx.x; q < n_q; q += blockDim.x) {
-        double acc = 0.0, c = 1.0, s = 0.0;
-        for (int t = 1; t < n_t; ++t) {
-            if ((t & 31) == 0) {
-                sincos(th * t, &s, &c);
-            } else {
-                const double c2 = c * cr - s * sr;
-                s = s * cr + c * sr;
-                c = c2;
-            }
-            acc = fma(v[t] * S[(int64_t)t * n_q + q], c, acc);
+    for (int t0 = 32 * threadIdx.x; t0 < n_t; t0 += 32 * blockDim.x) {
+        double c = 1.0, s = 0.0;
+        if (t0 > 0) sincos(th * t0, &s, &c);
+        for (int t = t0; t < t0 + 32 && t < n_t; ++t) {
+            ct[t] = c;
+            const double c2 = c * cr - s * sr;
+            s = s * cr + c * sr;
+            c = c2;
         }
+    }
+    __syncthreads();
+    for (int q = threadIdx.x; q < n_q; q += blockDim.x) {
+        double acc = 0.0;
+#pragma unroll 8
+        for (int t = 1; t < n_t; ++t) acc = fma(v[t] * S[(int64_t)t * n_q + q], ct[t], acc);
         Sqw[(int64_t)k * n_q + q] = dt * (v[0] * S[q] + 2.0 * acc);
     }
 }
@@ -61,8 +67,12 @@ int asd_sq_omega(const double *S, int n_t, int n_q, double dt, int window, doubl
     ASD_CHECK_ARG(dt > 0.0, "dt > 0");
     ASD_CHECK_ARG(window >= 0 && window <= 2, "window: 0 none, 1 Hann, 2 Gaussian");
     ASD_CHECK_ARG(window != 2 || width > 0.0, "Gaussian window needs width > 0");
-    sq_omega_kernel<<<n_w, 128, sizeof(double) * n_t, (cudaStream_t)stream>>>(
-        S, n_t, n_q, dt, window, width, omega, Sqw);
+    const size_t smem = 2 * sizeof(double) * (size_t)n_t;   // 96 KB at most
+    if (smem > 48 * 1024)
+        ASD_CUDA_TRY(cudaFuncSetAttribute(sq_omega_kernel,
+                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    sq_omega_kernel<<<n_w, 128, smem, (cudaStream_t)stream>>>(S, n_t, n_q, dt, window, width, omega,
+                                                              Sqw);
     ASD_CUDA_TRY(cudaGetLastError());
     return ASD_OK;
 }
