@@ -869,21 +869,6 @@ __device__ __forceinline__ float warp_max(float x)
     return x;
 }
 
-// K block of a work item before which sub-pass g (of G) of the previous item's phase
-// product is loaded and issued.  A sub-pass is one W stage (64 columns of one pass, the
-// pass's kWStages sub-passes in order).  The epilogue needs the first part of the item to
-// bin and convert the previous tile (the first sub-pass waits for that), the rest of it
-// to read the product out before the accumulator is needed again.  Sub-passes go in from
-// kSlotLo / kSlotDen of the item, evenly spaced up to kSlotHi / kSlotDen.  Measured on the
-// 32^3 glass (bins + 64 q, one pass of 3 sub-passes): all at 2/3 of the item 95.0 ms;
-// spread over [1/2, 5/6] 102.0, [1/3, 2/3] 101.4, [1/2, 1] 107.6, [1/6, 5/6] 112.1: the
-// binning of the previous tile sets the earliest slot, the read-out the latest.
-constexpr int kSlotLo = 2, kSlotHi = 2, kSlotDen = 3;
-__device__ __forceinline__ int phase_slot(int g, int nk, int G)
-{
-    return (nk * kSlotLo) / kSlotDen + (g * nk * (kSlotHi - kSlotLo)) / (kSlotDen * G);
-}
-
 // ------------------------------------------------------------------------------------
 // the kernel
 // ------------------------------------------------------------------------------------
@@ -1031,10 +1016,8 @@ __global__ void __launch_bounds__(tc_threads(BN, EW), 1) pc_tc_kernel(const __gr
             uint32_t phase = 0;
             bool ok = true;
             WorkCursor cu;
-            // the previous work item, while its phase sub-passes are still to be loaded:
-            // they go in among this item's K blocks (sub-pass g before block
-            // phase_slot(g)), so the phase product of item v - 1 runs while item v's MMAs
-            // run
+            // the previous work item, while its phase sub-passes are still to be loaded: they
+            // follow this item's K blocks
             int pend_p = -1, pend_n0 = 0, pend_G = 0;
             int64_t n_claimed = 0;  // work items claimed (static schedule)
             auto next_stage = [&]() {
@@ -1137,18 +1120,7 @@ __global__ void __launch_bounds__(tc_threads(BN, EW), 1) pc_tc_kernel(const __gr
                 // sample and K block inside it, and the operand window of that sample
                 int s = kg0 / wc.nkb, kb = kg0 - s * wc.nkb;
                 int xw = s * wc.F3 + 3 * ti.t, c = xw % wc.n_copies;
-                int g = 0;
                 for (int kg = kg0; kg < kg1 && ok; ++kg) {
-                    if constexpr (kPhaseOK) {
-                        while (pend_p >= 0 && g < pend_G &&
-                               kg - kg0 == phase_slot(g, nk, pend_G)) {
-                            if (!load_sub(g++)) {
-                                ok = false;
-                                break;
-                            }
-                        }
-                        if (!ok) break;
-                    }
                     if (!mbar_wait(empty0 + 8 * stage, phase ^ 1, args.err, DEV_TIMEOUT_TMA)) {
                         ok = false;
                         break;
@@ -1182,6 +1154,10 @@ __global__ void __launch_bounds__(tc_threads(BN, EW), 1) pc_tc_kernel(const __gr
                     }
                     if (kg == kg_take) take();
                 }
+                // the previous item's phase sub-passes, in the order the MMA thread issues them
+                if constexpr (kPhaseOK)
+                    if (pend_p >= 0)
+                        for (int g = 0; g < pend_G && ok; ++g) ok = load_sub(g);
                 pend_p = -1;
                 if (kPhaseOK && wc.npass > 0) {
                     pend_p = p_cur;
@@ -1313,17 +1289,7 @@ __global__ void __launch_bounds__(tc_threads(BN, EW), 1) pc_tc_kernel(const __gr
                 rel[acc] = phs ? 2 : 1;
                 tc_after();
                 const uint32_t d = tmem + acc * BN;
-                int g = 0;
                 for (int kb = 0; kb < nk; ++kb) {  // 0: the first block of this chunk
-                    if constexpr (kPhaseOK) {
-                        while (pend_acc >= 0 && g < pend_G && kb == phase_slot(g, nk, pend_G)) {
-                            if (!issue_sub(g++)) {
-                                ok = false;
-                                break;
-                            }
-                        }
-                        if (!ok) break;
-                    }
                     if (!mbar_wait(full0 + 8 * stage, phase, args.err, DEV_TIMEOUT_MMA)) {
                         ok = false;
                         break;
@@ -1354,6 +1320,15 @@ __global__ void __launch_bounds__(tc_threads(BN, EW), 1) pc_tc_kernel(const __gr
                 }
                 if (!ok) break;
                 commit_both(tfull0 + 8 * acc);
+                // The previous item's phase product, after this item's accumulator is handed
+                // over: its wait for the epilogue's BF16 copy then holds nobody up, where two
+                // thirds into the K blocks it stalled the rest of them (and so the epilogue's
+                // next tile) whenever the binning was the slower side.  48^3 glass BF16 at
+                // 2/3, 5/6 and the end: 103.0, 96.9, 94.0 ms; 32^3 glass split-BF16 the same.
+                if constexpr (kPhaseOK)
+                    if (pend_acc >= 0)
+                        for (int g = 0; g < pend_G && ok; ++g) ok = issue_sub(g);
+                if (!ok) break;
                 pend_acc = -1;
                 if (phs) {
                     // one pass: P sums the tile's chunks and is read out after the last
