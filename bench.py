@@ -394,8 +394,8 @@ def run_ours(args, W, ws, rank, local):
     if extra_pk:
         roof["measured_peaks"] = extra_pk
 
-    # per step: LL frame 0 + 4 RK4 stages per step, prep B + prep A copies (the FP32 form
-    # prepares B only), the fused contraction, normalisation (the memsets are torch's)
+    # per step: the LL run (one launch per 4096 steps), the operand preparation, the fused
+    # contraction, normalisation (the memsets are torch's)
     per_step = -(-(F - 1) // 4096) + 1 + 1 + 1
     out = {"metric": METRIC, "value": value, "unit": "TFLOP/s", "n_gpus": ws, "steps": args.steps,
            "warmup": args.warmup, "ms_per_step": t_step * 1e3, "higher_is_better": True,

@@ -28,10 +28,10 @@ namespace {
 
 constexpr int TM = 128, TN = 128, TK = 16;
 constexpr int kStages = 3;
-constexpr int kStageFloats = TK * (TM + TN);   // A twice, B
+constexpr int kStageFloats = TK * (TM + TN);   // A, B
 
 struct SimtParams {
-    const float *A;  // [R][ld], every value twice
+    const float *A;   // [S*F3][ld]: the trajectory by K
     const float *B;   // [S*Kseg][ld]
     int64_t ld;       // sites, padded to whole tiles
     int F3;
@@ -41,7 +41,7 @@ struct SimtParams {
     int N;
     int row_begin, row_end;
     int t_begin;      // displacement of grid slice blockIdx.z = 0
-    int a16;          // A rows start on 16 bytes (an even first row)
+    int a16;          // A rows start on 16 bytes (a first row that is a multiple of four)
     int warp_bins;    // per-warp FP32 bin copies after the FP64 arrays
     EpiParams e;
     int *err;         // device error word (index checks of a checked build)

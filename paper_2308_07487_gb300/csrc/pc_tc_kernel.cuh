@@ -123,13 +123,13 @@ __device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity)
     return ok != 0;
 }
 
-// (Inlined: as a call its saved registers were spilled around every wait of every role; 48^3
-// glass BF16 94.0 -> 84.1 ms, 32^3 glass split-BF16 19.3 -> 18.8 ms.)
 // Bounded wait for the phase with the given parity; false after kTimeoutNs (the error
 // word then holds `code`).  (A CTA pair's waits on barriers the other CTA signals use the
 // same test: the tcgen05 fences around the arrive and the wait order the tensor-memory
 // accesses, and TMA and MMA completions are counted by the barrier itself; a cluster-scope
-// acquire in every wait measured 30 % slower.)
+// acquire in every wait measured 30 % slower.)  Inlined: as a call its saved registers were
+// spilled around every wait of every role; 48^3 glass BF16 94.0 -> 84.1 ms, 32^3 glass
+// split-BF16 19.3 -> 18.8 ms.
 __device__ __forceinline__ bool mbar_wait_for(uint32_t bar, uint32_t parity, int *err, int code,
                                           unsigned long long limit_ns)
 {
