@@ -12,8 +12,10 @@
 // A stage needs every neighbour's previous stage.  Routes, by size (ll_run):
 //   ll_persistent<LOCAL>   one block per sample, the state in shared memory, a block barrier
 //                          between stages: samples of up to 2048 sites;
-//   ll_persistent<global>  a cooperative launch over every (sample, site), the state in L2,
-//                          a grid barrier between stages: up to four sites per thread;
+//   ll_tagged              a cooperative launch over every (sample, site), one site per thread;
+//                          blocks exchange stage inputs as words that carry their stage number;
+//   ll_persistent<global>  a cooperative launch, the state in L2, a grid barrier between stages:
+//                          up to four sites per thread;
 //   rk4_stage              one launch per stage: larger systems.
 // The last stage writes the new state and, every `stride` steps, the trajectory frame in the
 // site-major layout traj[i][s][f][a] consumed by asd_pair_corr.  All routes do the same
@@ -135,7 +137,8 @@ struct LLRun {
     const float *in;     // [S][N][3] state at the first step
     float *out;          // [S][N][3] state after the last step, or null
     float4 *Y, *T1, *T2; // global route: state and stage inputs [S][N]
-    unsigned *bar;       // global route: grid barrier count (zero at launch)
+    int n_buf;           // ll_tagged: stage inputs from Y on, 2 .. kLLMaxBufs
+    unsigned *bar;       // cooperative routes: grid barrier count (zero at launch)
     float *traj;
     int F;
     int64_t step0, step1;  // steps [step0, step1) of the run
@@ -144,6 +147,7 @@ struct LLRun {
     int stage_frames;    // 1: frames go out through shared memory, kLLFrames at a time
     int *err;
 };
+constexpr int kLLMaxBufs = 9;                       // stage inputs of ll_tagged
 constexpr int kLLFrames = 4;
 constexpr int kLLFramePitch = 3 * kLLFrames + 1;   // words per site (odd: no bank conflicts)
 
@@ -157,7 +161,7 @@ constexpr int kLLFramePitch = 3 * kLLFrames + 1;   // words per site (odd: no ba
 // (4.1 -> 0.32 us per stage); 64^3, 159 steps, 6.14 -> 3.36 ms (9.6 -> 5.3 us per stage, of
 // which the barrier about 2); frames stored by each site as they come instead of gathered:
 // 130 us and 3.78 ms.  36^2 sites and two samples, 90 steps: 1.58 -> 0.53 ms, though only
-// two blocks run (the grid route's stage takes 2.4 us at any size up to 50 thousand sites).
+// two blocks run.
 template <int SPT, int Z, bool LOCAL>
 __global__ void __launch_bounds__(kLLThreads, 1) ll_persistent(const __grid_constant__ LLRun r)
 {
@@ -341,6 +345,213 @@ __global__ void __launch_bounds__(kLLThreads, 1) ll_persistent(const __grid_cons
             }
 }
 
+// 16-byte loads and stores of one access at GPU scope: a value and its stage number together.
+__device__ __forceinline__ float4 ld_tagged(const float4 *p)
+{
+    uint64_t lo, hi;
+    asm volatile("{\n\t.reg .b128 t;\n\tld.relaxed.gpu.global.b128 t, [%2];\n\t"
+                 "mov.b128 {%0, %1}, t;\n}\n"
+                 : "=l"(lo), "=l"(hi)
+                 : "l"(p)
+                 : "memory");
+    return make_float4(__uint_as_float((uint32_t)lo), __uint_as_float((uint32_t)(lo >> 32)),
+                       __uint_as_float((uint32_t)hi), __uint_as_float((uint32_t)(hi >> 32)));
+}
+__device__ __forceinline__ void st_tagged(float4 *p, float3 v, int tag)
+{
+    const uint64_t lo = (uint64_t)__float_as_uint(v.x) | (uint64_t)__float_as_uint(v.y) << 32;
+    const uint64_t hi = (uint64_t)__float_as_uint(v.z) | (uint64_t)(uint32_t)tag << 32;
+    asm volatile("{\n\t.reg .b128 t;\n\tmov.b128 t, {%1, %2};\n\t"
+                 "st.relaxed.gpu.global.b128 [%0], t;\n}\n" ::"l"(p), "l"(lo), "l"(hi)
+                 : "memory");
+}
+
+// The same run, one site per thread, without a grid barrier in every stage (which was about 2
+// of the 2.5 to 2.8 us of a stage at these sizes).  The block's own stage inputs are in shared
+// memory; other blocks' come from global memory as 16-byte words that carry their stage number,
+// and a reader waits for the number it needs, so a stage costs one store and one load through
+// L2.  Stage g's inputs are in buffer g mod n_buf; a grid barrier every n_buf - 1 stages keeps a
+// block from overwriting a buffer that another still reads, whatever the bond table.  A block
+// waits only for what others wrote in the stage before, so every wait ends; all are bounded.
+// Measured against a barrier per stage: 48^3 sites, 67 steps, 738 -> 566 us; 8 samples of 18^3, 105
+// steps, 1022 -> 736 us (2.1 and 1.75 us per stage).  With two sites per thread it is slower (64^3,
+// 159 steps, 3.35 -> 4.17 ms: a stage is bound by issue slots there, and the tests of the
+// numbers add to them), so ll_persistent keeps those.
+template <int Z>
+__global__ void __launch_bounds__(kLLThreads, 1) ll_tagged(const __grid_constant__ LLRun r)
+{
+    extern __shared__ __align__(16) uint8_t ll_smem[];
+    constexpr bool kReg = Z > 0;   // bonds in registers
+    const LLArgs &a = r.a;
+    const int N = (int)a.N, nt = blockDim.x, tid = threadIdx.x;
+    const int64_t n = (int64_t)N * a.S;
+    const int64_t g0 = (int64_t)blockIdx.x * nt;
+    // two stages' inputs of the block's sites, bonds [k][slot], held frames
+    float4 *sm = reinterpret_cast<float4 *>(ll_smem);
+    int *sm_nbr = reinterpret_cast<int *>(sm + 2 * nt);
+    float *sm_J = reinterpret_cast<float *>(sm_nbr + (kReg ? 0 : a.z * nt));
+    float *sm_frames = sm_J + (kReg ? 0 : a.z * nt);
+
+    constexpr int ZB = kReg ? Z : 1;
+    int nb[ZB];
+    float Jr[ZB];
+    const bool on = g0 + tid < n;
+    const int64_t gc = on ? g0 + tid : g0;
+    const int s = (int)(gc / N), site = (int)(gc - (int64_t)s * N);
+    // a neighbour as its slot, or -2 - its flattened index when another block has it (-1: none)
+    const int off = (int)((int64_t)s * N);
+    auto place = [&](int j) {
+        if (j < 0) return -1;
+        const int64_t slot = (int64_t)j + off - g0;
+        return slot >= 0 && slot < nt ? (int)slot : -2 - (j + off);
+    };
+    if (kReg) {
+#pragma unroll
+        for (int k = 0; k < ZB; ++k) {
+            nb[k] = on ? place(__ldg(a.nbr + (int64_t)site * Z + k)) : -1;
+            Jr[k] = on ? __ldg(a.J + (int64_t)site * Z + k) : 0.f;
+        }
+    } else if (on) {
+        for (int k = 0; k < a.z; ++k) {
+            sm_nbr[k * nt + tid] = place(__ldg(a.nbr + (int64_t)site * a.z + k));
+            sm_J[k * nt + tid] = __ldg(a.J + (int64_t)site * a.z + k);
+        }
+    }
+    const float *src = r.in + 3 * gc;
+    float3 y = make_float3(src[0], src[1], src[2]), x = y, acc;
+    float *dst = r.traj + (((int64_t)site * a.S + s) * r.F + r.step0 / r.stride) * 3;
+    if (on) {
+        sm[tid] = make_float4(y.x, y.y, y.z, 0.f);
+        st_tagged(r.Y + gc, y, 0);
+        for (int b = 1; b < r.n_buf; ++b) st_tagged(r.Y + b * n + gc, y, -1);
+        if (r.step0 == 0) {
+            dst[0] = y.x; dst[1] = y.y; dst[2] = y.z;
+        }
+    }
+    int in_frame = (int)(r.step0 % r.stride);   // steps since the last frame
+    int n_held = 0;                             // frames held (as in ll_persistent)
+    int64_t f_held = r.step0 / r.stride + 1;
+    auto put_frames = [&]() {
+        __syncthreads();
+        const int words = 3 * n_held, left = (int)min((int64_t)nt, n - g0);
+        for (int e = tid; e < left * words; e += nt) {
+            const int slot = e / words, c = e - slot * words;
+            const int64_t g = g0 + slot, sl = g / N, i = g - sl * N;
+            r.traj[((i * a.S + sl) * r.F + f_held) * 3 + c] = sm_frames[slot * kLLFramePitch + c];
+        }
+        f_held += n_held;
+        n_held = 0;
+        __syncthreads();
+    };
+    unsigned target = gridDim.x;
+    if (!grid_barrier(r.bar, target, r.err)) return;
+
+    bool alive = true;   // no wait of this thread has given up
+    // the value of stage g of another block's site, once it is there
+    auto wait_tagged = [&](const float4 *p, int g) {
+        float4 v = ld_tagged(p);
+        unsigned long long t0 = 0;
+        for (unsigned it = 1; __float_as_int(v.w) != g; ++it) {
+            if ((it & 1023u) == 0) {
+                unsigned long long now;
+                asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
+                if (t0 == 0) t0 = now;
+                else if (now - t0 > kGridTimeoutNs) {
+                    atomicCAS(r.err, 0, (int)DEV_TIMEOUT_GRID);
+                    alive = false;
+                    break;
+                }
+            }
+            v = ld_tagged(p);
+        }
+        return v;
+    };
+    // derivative of the own site from the inputs of stage g (V: the block's, G: everyone's)
+    auto deriv = [&](int g, const float4 *V, const float4 *G) {
+        float3 h = make_float3(0.f, 0.f, -a.Hz);
+        if (kReg) {
+            // all neighbours' loads in flight, then the late ones again, then the sums in bond
+            // order
+            float4 sj[ZB];
+#pragma unroll
+            for (int k = 0; k < ZB; ++k) {
+                if (nb[k] >= -1) sj[k] = V[nb[k] < 0 ? tid : nb[k]];
+                else sj[k] = ld_tagged(G - (nb[k] + 2));
+            }
+#pragma unroll
+            for (int k = 0; k < ZB; ++k)
+                if (nb[k] < -1 && __float_as_int(sj[k].w) != g)
+                    sj[k] = wait_tagged(G - (nb[k] + 2), g);
+#pragma unroll
+            for (int k = 0; k < ZB; ++k)
+                if (nb[k] != -1)
+                    add_bond(h, Jr[k], sj[k].x, sj[k].y, sj[k].z,
+                             a.D ? a.D + ((int64_t)site * Z + k) * 3 : nullptr);
+        } else {
+            for (int k = 0; k < a.z; ++k) {
+                const int j = sm_nbr[k * nt + tid];
+                if (j == -1) continue;
+                const float4 sj = j >= 0 ? V[j] : wait_tagged(G - (j + 2), g);
+                add_bond(h, sm_J[k * nt + tid], sj.x, sj.y, sj.z,
+                         a.D ? a.D + ((int64_t)site * a.z + k) * 3 : nullptr);
+            }
+        }
+        h.z = fmaf(-2.f * a.A, x.z, h.z);
+        return cross(h, x);
+    };
+    int g = 0, b_in = 0, since = 0;   // stage, its buffer, stages since the last grid barrier
+    for (int64_t st = r.step0; st < r.step1; ++st) {
+#pragma unroll
+        for (int stage = 1; stage <= 4; ++stage) {
+            const float4 *V = sm + (stage & 1 ? 0 : nt), *G = r.Y + (int64_t)b_in * n;
+            float4 *out = sm + (stage & 1 ? nt : 0);
+            if (++b_in == r.n_buf) b_in = 0;
+            if (on) {
+                const float3 k = deriv(g, V, G);
+                if (stage == 1) {
+                    acc = k;
+                } else if (stage < 4) {
+                    acc.x += 2.f * k.x;
+                    acc.y += 2.f * k.y;
+                    acc.z += 2.f * k.z;
+                }
+                if (stage < 4) {
+                    const float c = stage == 3 ? r.dt : 0.5f * r.dt;
+                    x = make_float3(fmaf(c, k.x, y.x), fmaf(c, k.y, y.y), fmaf(c, k.z, y.z));
+                } else {
+                    const float c = r.dt / 6.f;
+                    y = make_float3(fmaf(c, acc.x + k.x, y.x), fmaf(c, acc.y + k.y, y.y),
+                                    fmaf(c, acc.z + k.z, y.z));
+                    x = y;
+                }
+                st_tagged(r.Y + (int64_t)b_in * n + gc, x, g + 1);
+                out[tid] = make_float4(x.x, x.y, x.z, 0.f);
+            }
+            ++g;
+            if (stage == 4 && ++in_frame == r.stride) {
+                in_frame = 0;
+                dst += 3;
+                float *d = r.stage_frames ? sm_frames + tid * kLLFramePitch + 3 * n_held : dst;
+                if (on) {
+                    d[0] = y.x; d[1] = y.y; d[2] = y.z;
+                }
+                if (r.stage_frames && ++n_held == kLLFrames) put_frames();
+            }
+            if (!__syncthreads_and(alive)) return;
+            if (++since == r.n_buf - 1) {
+                since = 0;
+                target += gridDim.x;
+                if (!grid_barrier(r.bar, target, r.err)) return;
+            }
+        }
+    }
+    if (n_held > 0) put_frames();
+    if (r.out && on) {
+        float *o = r.out + 3 * gc;
+        o[0] = y.x; o[1] = y.y; o[2] = y.z;
+    }
+}
+
 typedef void (*LLKernel)(LLRun);
 
 template <int SPT, bool LOCAL>
@@ -355,7 +566,7 @@ LLKernel ll_kernel_z(int z)
 // the system is too large for one.
 struct LLRoute {
     LLKernel k = nullptr;
-    bool local = false;
+    bool local = false, tagged = false;
     unsigned grid = 0, block = 0;
     size_t smem = 0;
     bool stage_frames = false;
@@ -408,9 +619,13 @@ int ll_route(const LLArgs &a, LLRoute *out)
         r.grid = (unsigned)((n + (int64_t)r.block * spt - 1) / ((int64_t)r.block * spt));
         r.smem = bonds(spt, (int64_t)spt * r.block);
         if (r.smem > kLLMaxSmem) return ASD_OK;
-        add_frames(r, r.smem, (int64_t)spt * r.block);
-        r.k = spt == 1 ? ll_kernel_z<1, false>(a.z)
-                       : spt == 2 ? ll_kernel_z<2, false>(a.z) : ll_kernel_z<4, false>(a.z);
+        // one site per thread: ll_tagged, unless many bonds leave no room for its inputs
+        const size_t own = 2 * sizeof(float4) * (size_t)r.block;
+        r.tagged = spt == 1 && r.smem + own <= kLLMaxSmem;
+        add_frames(r, r.smem + (r.tagged ? own : 0), (int64_t)spt * r.block);
+        r.k = r.tagged ? (a.z == 4 ? ll_tagged<4> : a.z == 6 ? ll_tagged<6> : ll_tagged<0>)
+              : spt == 1 ? ll_persistent<1, 0, false>
+              : spt == 2 ? ll_kernel_z<2, false>(a.z) : ll_kernel_z<4, false>(a.z);
         ASD_CUDA_TRY(cudaFuncSetAttribute(r.k, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                           (int)r.smem));
         int per_sm = 0;
@@ -422,10 +637,11 @@ int ll_route(const LLArgs &a, LLRoute *out)
     return ASD_OK;
 }
 
-// The whole run with the work buffers at ws (48 bytes per site-sample, 16-byte aligned) and
-// the barrier count at bar.
+// The whole run with the work buffers at ws (16-byte aligned, ws_bytes >= 48 per site-sample)
+// and the barrier count at bar.
 int ll_run(const LLArgs &a, const LLRoute &rt, const float *spins0, float dt, int n_frames,
-           int stride, float *traj, float *spins_out, void *ws, unsigned *bar, cudaStream_t s)
+           int stride, float *traj, float *spins_out, void *ws, size_t ws_bytes, unsigned *bar,
+           cudaStream_t s)
 {
     const int64_t n = a.N * a.S;
     const int64_t steps = (int64_t)(n_frames - 1) * stride;
@@ -435,6 +651,14 @@ int ll_run(const LLArgs &a, const LLRoute &rt, const float *spins0, float dt, in
         r.Y = static_cast<float4 *>(ws);
         r.T1 = r.Y + n;
         r.T2 = r.T1 + n;
+        // (the state between launches goes through the first 12 bytes per site of T1, or of a
+        // part of the work area that ll_tagged does not use)
+        float *mid = reinterpret_cast<float *>(r.T1);
+        if (rt.tagged) {
+            const int keep = steps > kLLStepsPerLaunch ? 1 : 0;
+            r.n_buf = (int)std::min<size_t>(kLLMaxBufs, ws_bytes / (sizeof(float4) * n) - keep);
+            mid = reinterpret_cast<float *>(r.Y + (int64_t)r.n_buf * n);
+        }
         r.bar = bar;
         r.traj = traj;
         r.F = n_frames;
@@ -449,8 +673,7 @@ int ll_run(const LLArgs &a, const LLRoute &rt, const float *spins0, float dt, in
             r.step0 = st;
             r.step1 = std::min<int64_t>(steps, st + kLLStepsPerLaunch);
             r.in = in;
-            // between launches the state goes through the first 12 bytes per site of T1
-            r.out = r.step1 == steps ? spins_out : reinterpret_cast<float *>(r.T1);
+            r.out = r.step1 == steps ? spins_out : mid;
             if (rt.local) {
                 rt.k<<<rt.grid, rt.block, rt.smem, s>>>(r);
                 ASD_CUDA_TRY(cudaGetLastError());
@@ -509,9 +732,9 @@ extern "C" int asd_ll_integrate(const asd_system *sys, int n_samples, const floa
     char *ws = nullptr;
     // (a block per sample in one launch keeps everything on chip)
     const bool need = !rt.local || (int64_t)(n_frames - 1) * stride > kLLStepsPerLaunch;
-    const size_t bytes = 48 * (size_t)n;
+    const size_t bytes = (rt.tagged ? 16 * (kLLMaxBufs + 1) : 48) * (size_t)n;
     if (need) ASD_CUDA_TRY(cudaMallocAsync(&ws, bytes + 16, s));
-    rc = ll_run(a, rt, spins0, dt, n_frames, stride, traj, spins_out, ws,
+    rc = ll_run(a, rt, spins0, dt, n_frames, stride, traj, spins_out, ws, bytes,
                 reinterpret_cast<unsigned *>(ws + bytes), s);
     if (need) cudaFreeAsync(ws, s);
     return rc;
@@ -618,6 +841,7 @@ extern "C" int asd_ll_integrate_noalloc(const asd_system *sys, int n_samples, co
     rc = ll_route(a, &rt);
     if (rc) return rc;
     return ll_run(a, rt, spins0, dt, n_frames, stride, traj, spins_out, ws,
+                  sizeof(float) * 4 * 3 * (size_t)kLLStaticMaxSiteSamples,
                   reinterpret_cast<unsigned *>(ws + 4 * 3 * kLLStaticMaxSiteSamples),
                   (cudaStream_t)stream);
 }
