@@ -346,7 +346,7 @@ int asd_ll_integrate(const asd_system *sys, int n_samples, const float *spins0, 
  * begins.  The address is looked up again when the device's context has changed (after
  * a cudaDeviceReset, for instance).  All calls share the one array: calls whose work can
  * overlap on the GPU (on different streams without ordering) race on it and give wrong
- * results; calls on one stream are safe.  Nothing in the array needs to start at zero: every buffer is fully
+ * results or ASD_ETIMEOUT; calls on one stream are safe.  Nothing in the array needs to start at zero: every buffer is fully
  * written before it is read.  Allocates nothing (no cudaMalloc, cudaMallocAsync or
  * cudaFree).
  */
