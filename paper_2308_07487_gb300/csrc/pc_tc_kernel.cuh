@@ -932,20 +932,26 @@ __global__ void __launch_bounds__(tc_threads(BN, EW), 1) pc_tc_kernel(const __gr
     const EpiLayout EL = epi_layout(args.VB, args.NB, args.NQ, BN, EW, args.det);
     uint64_t *bars = reinterpret_cast<uint64_t *>(epi + EL.total);
     // bars: full[stages], empty[stages], tfull[2], tempty[2], drain, wqfull[kWQ],
-    // wqempty[kWQ], conv, pfull, pempty, tmm[2], gfull[2], gempty[2]; then the work ring
+    // wqempty[kWQ], conv[2], pfull, pempty, tmm[2], gfull[2], gempty[2]; then the work ring
     // wq[kWQ] and the TMEM address slot
     const uint32_t wqfull0 = saddr(bars + 2 * stages + 5);
     const uint32_t wqempty0 = saddr(bars + 2 * stages + 5 + kWQ);
-    // conv: the epilogue has stored a chunk's G as BF16 hi / lo (one arrival per warp);
+    // conv[a]: the epilogue has stored the G of the chunk in accumulator a as BF16 hi / lo (one
+    // arrival per warp).  One barrier per accumulator: the MMA thread hands out the next item's
+    // accumulator before it waits for this item's conversion, so the epilogue may convert two
+    // items before the first wait; on one barrier the second phase would complete unseen and
+    // the wait for the first (by parity) never end.  A second arrival on conv[a] needs the
+    // accumulator again, which the MMA thread hands out only after tmm[a], issued after its
+    // wait on conv[a];
     // pfull: the phase product to be read out is complete; pempty: the read-out warps have
     // read it; tmm[a]: the phase product of the chunk in accumulator a is complete, so the
     // buffer is free (for phase work the MMA thread releases the accumulator, not the
     // epilogue); gfull / gempty: a tile's geometry buffer is filled / has been used
-    const uint32_t conv = saddr(bars + 2 * stages + 5 + 2 * kWQ);
-    const uint32_t pfull = conv + 8, pempty = conv + 16, tmm0 = conv + 24;
-    const uint32_t gfull0 = conv + 40, gempty0 = conv + 56;
+    const uint32_t conv0 = saddr(bars + 2 * stages + 5 + 2 * kWQ);
+    const uint32_t pfull = conv0 + 16, pempty = conv0 + 24, tmm0 = conv0 + 32;
+    const uint32_t gfull0 = conv0 + 48, gempty0 = conv0 + 64;
     volatile WorkSlot *wq = reinterpret_cast<volatile WorkSlot *>(
-        (reinterpret_cast<uintptr_t>(bars + 2 * stages + 14 + 2 * kWQ) + 15) & ~(uintptr_t)15);
+        (reinterpret_cast<uintptr_t>(bars + 2 * stages + 15 + 2 * kWQ) + 15) & ~(uintptr_t)15);
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(const_cast<WorkSlot *>(wq + kWQ));
     const uint32_t full0 = saddr(bars), empty0 = saddr(bars + stages);
     const uint32_t tfull0 = saddr(bars + 2 * stages), tempty0 = saddr(bars + 2 * stages + 2);
@@ -976,12 +982,11 @@ __global__ void __launch_bounds__(tc_threads(BN, EW), 1) pc_tc_kernel(const __gr
             // epilogue and read-out warp and the geometry warp
             mbar_init(wqempty0 + 8 * k, (leader ? 1 : 0) + kEpiWarps + 1 + kRoWarps);
         }
-        mbar_init(conv, kEpiWarps * CG);
         mbar_init(pfull, 1);
         mbar_init(pempty, 4 * CG);
-        mbar_init(tmm0, 1);
-        mbar_init(tmm0 + 8, 1);
         for (int a = 0; a < 2; ++a) {
+            mbar_init(conv0 + 8 * a, kEpiWarps * CG);
+            mbar_init(tmm0 + 8 * a, 1);
             mbar_init(gfull0 + 8 * a, 1);
             mbar_init(gempty0 + 8 * a, kEpiWarps);
         }
@@ -1206,8 +1211,9 @@ __global__ void __launch_bounds__(tc_threads(BN, EW), 1) pc_tc_kernel(const __gr
             // completes P for the read-out
             int pend_acc = -1, pend_G = 0;
             bool pend_add = false, pend_done = false;
-            // converted chunks waited for; passes that started P afresh (one read-out each)
-            uint32_t n_conv = 0, n_own = 0;
+            // parity of the next conversion to wait for, one bit per accumulator; passes that
+            // started P afresh (one read-out each)
+            uint32_t conv_par = 0, n_own = 0;
             // how each accumulator was last released (0: not used yet, 1: by the epilogue
             // on tempty, 2: by this thread's commit on tmm after the chunk's phase product)
             // and the waits taken on each barrier
@@ -1225,9 +1231,12 @@ __global__ void __launch_bounds__(tc_threads(BN, EW), 1) pc_tc_kernel(const __gr
                 if (j == 0) {
                     // G stored as BF16 by the epilogue (once per chunk); a pass that starts
                     // P afresh waits until the previous P has been read out
-                    if (pp == 0 &&
-                        !mbar_wait(conv, n_conv++ & 1, args.err, DEV_TIMEOUT_MMA))
-                        return false;
+                    if (pp == 0) {
+                        if (!mbar_wait(conv0 + 8 * pend_acc, (conv_par >> pend_acc) & 1,
+                                       args.err, DEV_TIMEOUT_MMA))
+                            return false;
+                        conv_par ^= 1u << pend_acc;
+                    }
                     if (!pend_add) {
                         if (!mbar_wait(pempty, (n_own & 1) ^ 1, args.err, DEV_TIMEOUT_MMA))
                             return false;
@@ -1959,7 +1968,7 @@ __global__ void __launch_bounds__(tc_threads(BN, EW), 1) pc_tc_kernel(const __gr
             __syncwarp();
             // (a pair's epilogue warps arrive on the first CTA's barriers)
             if (lane == 0) {
-                const uint32_t a = ph ? conv : tempty0 + 8 * acc;
+                const uint32_t a = (ph ? conv0 : tempty0) + 8 * acc;
                 if constexpr (CG == 2) mbar_arrive_cl(lead(a));
                 else mbar_arrive(a);
             }
