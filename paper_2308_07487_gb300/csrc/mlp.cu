@@ -112,15 +112,17 @@ __device__ __forceinline__ void tile_backward(float (&acc)[4][4], const float *w
     }
 }
 
-// A layer's BF16 weights [rows][cols] as FP32 rows of `ld` floats, eight at a time where the
-// caller's pointer is 16-byte aligned and a row is whole words.
+// A layer's BF16 weights [rows][cols] as FP32 rows of `ld` floats (zeros past a row's end), eight
+// at a time where the caller's pointer is 16-byte aligned and no eight cross a gap between rows
+// (rows * cols is a multiple of eight); else one by one, from any address.
 __device__ __forceinline__ void load_weights(float *dst, int ld, const __nv_bfloat16 *src, int rows,
                                              int cols, int t, int nt)
 {
-    if (cols % 8 == 0 && (reinterpret_cast<uintptr_t>(src) & 15) == 0) {
+    const bool dense = ld == cols;
+    if ((dense || cols % 8 == 0) && (reinterpret_cast<uintptr_t>(src) & 15) == 0) {
         for (int e = t; e < rows * cols / 8; e += nt) {
             const uint4 v = __ldg(reinterpret_cast<const uint4 *>(src) + e);
-            const int r = 8 * e / cols, c = 8 * e - r * cols;
+            const int i = 8 * e;
             const uint32_t u[4] = {v.x, v.y, v.z, v.w};
             float4 f[2];
             float *fp = reinterpret_cast<float *>(f);
@@ -129,7 +131,7 @@ __device__ __forceinline__ void load_weights(float *dst, int ld, const __nv_bflo
                 fp[2 * k] = __uint_as_float(u[k] << 16);
                 fp[2 * k + 1] = __uint_as_float(u[k] & 0xffff0000u);
             }
-            float4 *o = reinterpret_cast<float4 *>(dst + r * ld + c);
+            float4 *o = reinterpret_cast<float4 *>(dst + (dense ? i : i / cols * ld + i % cols));
             o[0] = f[0];
             o[1] = f[1];
         }
@@ -198,13 +200,9 @@ __global__ void __launch_bounds__(kLG) loss_grad_kernel(MlpView net, int64_t n,
     float *DO = Ds + DEPTH * H * kAP;               // [4][kAP] outputs, then their deltas
 
     const int t = threadIdx.x, ty = t >> 4, tx = t & 15;
-    if (ninp == nin) {
-        load_weights(W1, nin, net.W1, 1, H * nin, t, kLG);
-    } else {
-        load_weights(W1, ninp, net.W1, H, nin, t, kLG);
-        for (int e = t; e < (ninp - nin) * kTile; e += kLG)
-            Xs[(nin + e / kTile) * kAP + e % kTile] = 0.f;
-    }
+    load_weights(W1, ninp, net.W1, H, nin, t, kLG);
+    for (int e = t; e < (ninp - nin) * kTile; e += kLG)   // the padding inputs
+        Xs[(nin + e / kTile) * kAP + e % kTile] = 0.f;
     load_weights(Wh, kWP, net.W2, H, H, t, kLG);
     if (DEPTH == 3) load_weights(Wh + (DEPTH - 2) * H * kWP, kWP, net.Wm, H, H, t, kLG);
     load_weights(W3, H, net.W3, 4, H, t, kLG);
