@@ -144,11 +144,13 @@ __device__ __forceinline__ void load_weights(float *dst, int ld, const __nv_bflo
 }
 
 // g[i][j] += sum over the tile's samples of d[k_i] v[c_j], k_i = ty + 16 i, c_j = tx + 16 j
-// (columns from n_c on are left out).
+// (columns from n_c on are left out).  The tile's 64 terms are summed by themselves and added
+// once: a running sum over all of a block's tiles would lose the small terms of later ones.
 __device__ __forceinline__ void tile_grad(float (&g)[4][4], const float *d, const float *v, int n_c,
                                           int ty, int tx)
 {
-#pragma unroll 2
+    float s[4][4] = {};
+#pragma unroll 4
     for (int m = 0; m < kTile; m += 4) {
         float4 a[4], b[4];
 #pragma unroll
@@ -163,10 +165,14 @@ __device__ __forceinline__ void tile_grad(float (&g)[4][4], const float *d, cons
 #pragma unroll
             for (int j = 0; j < 4; ++j)
                 if (16 * j < n_c)
-                    g[i][j] = fmaf(a[i].w, b[j].w,
+                    s[i][j] = fmaf(a[i].w, b[j].w,
                                    fmaf(a[i].z, b[j].z,
-                                        fmaf(a[i].y, b[j].y, fmaf(a[i].x, b[j].x, g[i][j]))));
+                                        fmaf(a[i].y, b[j].y, fmaf(a[i].x, b[j].x, s[i][j]))));
     }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) g[i][j] += s[i][j];
 }
 
 // Shared memory (floats) of the training kernel.
@@ -311,12 +317,14 @@ __global__ void __launch_bounds__(kLG) loss_grad_kernel(MlpView net, int64_t n,
         {
             const int q = t >> 6, c = t & 63;   // W3[q][c]
             const float *dq = DO + q * kAP, *hc = Hl + c * kAP;
+            float s = 0.f;
 #pragma unroll 4
             for (int m = 0; m < kTile; m += 4) {
                 const float4 d4 = *reinterpret_cast<const float4 *>(dq + m);
                 const float4 h4 = *reinterpret_cast<const float4 *>(hc + m);
-                g3 = fmaf(d4.w, h4.w, fmaf(d4.z, h4.z, fmaf(d4.y, h4.y, fmaf(d4.x, h4.x, g3))));
+                s = fmaf(d4.w, h4.w, fmaf(d4.z, h4.z, fmaf(d4.y, h4.y, fmaf(d4.x, h4.x, s))));
             }
+            g3 += s;
         }
         // biases: DEPTH x H hidden, then 4 outputs
 #pragma unroll
