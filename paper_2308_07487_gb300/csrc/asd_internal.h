@@ -99,6 +99,17 @@ constexpr int kBM = 128;            // rows (sites i) per tile = TMEM lanes
 constexpr int kMaxCopies = 8;       // shifted operand copies (16-byte TMA start rule)
 constexpr int kMaxProblems = 4096;  // batched work list
 constexpr size_t kMinSmem = 120 * 1024;  // tensor-core kernel: one CTA per SM
+constexpr size_t kMaxSmem = 232448;      // shared memory that a block can have
+
+// Lets a kernel's launches use up to `most` bytes of dynamic shared memory.  `most` is the same
+// number at every call for a kernel, not the size of the launch at hand: the limit belongs to
+// the kernel, and a thread that set a smaller one between another thread's call of this and its
+// launch would have that launch refused.
+template <typename Kernel>
+inline cudaError_t allow_smem(Kernel k, size_t most)
+{
+    return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+}
 constexpr int kLutMax = 16384;           // largest d2 -> bin table kept in shared memory
 constexpr int kQChunk = 16;              // q-vectors per chunk of the phase epilogue (cs
                                          // rows are zero padded to whole chunks)

@@ -604,8 +604,7 @@ int ll_route(const LLArgs &a, LLRoute *out)
             r.grid = (unsigned)a.S;
             r.block = (unsigned)(((a.N + spt - 1) / spt + 31) / 32 * 32);
             add_frames(r, smem, a.N);
-            ASD_CUDA_TRY(cudaFuncSetAttribute(r.k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              (int)r.smem));
+            ASD_CUDA_TRY(allow_smem(r.k, kLLMaxSmem));
             *out = r;
             return ASD_OK;
         }
@@ -626,8 +625,7 @@ int ll_route(const LLArgs &a, LLRoute *out)
         r.k = r.tagged ? (a.z == 4 ? ll_tagged<4> : a.z == 6 ? ll_tagged<6> : ll_tagged<0>)
               : spt == 1 ? ll_persistent<1, 0, false>
               : spt == 2 ? ll_kernel_z<2, false>(a.z) : ll_kernel_z<4, false>(a.z);
-        ASD_CUDA_TRY(cudaFuncSetAttribute(r.k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)r.smem));
+        ASD_CUDA_TRY(allow_smem(r.k, kLLMaxSmem));
         int per_sm = 0;
         ASD_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, r.k, (int)r.block,
                                                                    r.smem));

@@ -466,8 +466,7 @@ int mc_route(const MCArgs &a, const int64_t *off, int n_colors, int adapt, int s
         r.grid = (unsigned)a.S;
         r.block = (unsigned)std::min<int64_t>(1024, (widest + 31) / 32 * 32);
         r.smem = sizeof(float4) * (size_t)a.N;
-        ASD_CUDA_TRY(cudaFuncSetAttribute(r.k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)r.smem));
+        ASD_CUDA_TRY(allow_smem(r.k, sizeof(float4) * kMcLocalSites));
         *out = r;
         return ASD_OK;
     }
@@ -661,7 +660,7 @@ int launch_learned_t(const MCArgs &a, float *spins, int sms, cudaStream_t s)
 {
     auto k = mc_learned_kernel<NIN, T>;
     const size_t smem = ml_smem<NIN, T>(a.net.depth);
-    ASD_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    ASD_CUDA_TRY(allow_smem(k, ml_smem<NIN, T>(3)));
     const int64_t groups = (a.n_sites_c * a.S + T - 1) / T;
     const int64_t blocks = (groups + kMlBlock - 1) / kMlBlock;
     const int64_t most = 2 * (int64_t)sms;

@@ -492,7 +492,7 @@ int asd_mlp_loss_grad(const asd_mlp *net, int64_t n, const float *x, const float
     const int nin = net->n_in;
     const size_t smem = sizeof(float) * (size_t)lg_smem_floats(nin, depth);
     auto k = depth == 2 ? loss_grad_kernel<2> : loss_grad_kernel<3>;
-    ASD_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    ASD_CUDA_TRY(allow_smem(k, sizeof(float) * (size_t)lg_smem_floats(kMlpMaxIn, depth)));
     int dev = 0, sms = 0;
     ASD_CUDA_TRY(cudaGetDevice(&dev));
     ASD_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));

@@ -29,6 +29,7 @@ namespace {
 constexpr int TM = 128, TN = 128, TK = 16;
 constexpr int kStages = 3;
 constexpr int kStageFloats = TK * (TM + TN);   // A, B
+constexpr size_t kSumBytes = 48 * 1024;        // most that the bin and phase sums take
 
 struct SimtParams {
     const float *A;   // [S*F3][ld]: the trajectory by K
@@ -307,12 +308,11 @@ int launch_simt(asd_corr_plan *p, int64_t row_begin, int64_t row_end, int t_begi
         return ASD_EUNSUPPORTED;
     }
     size_t smem = sizeof(double) * (p->n_bins + p->n_q * p->q_parts);
-    // per-warp FP32 bin copies where they and the FP64 sums fit 48 KB
-    P.warp_bins = !p->d.deterministic && smem + sizeof(float) * 8 * p->n_bins <= 48 * 1024;
+    // per-warp FP32 bin copies where they and the FP64 sums fit
+    P.warp_bins = !p->d.deterministic && smem + sizeof(float) * 8 * p->n_bins <= kSumBytes;
     if (P.warp_bins) smem += sizeof(float) * 8 * p->n_bins;
     smem += sizeof(float) * kStages * kStageFloats;
-    ASD_CUDA_TRY(cudaFuncSetAttribute(simt_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)smem));
+    ASD_CUDA_TRY(allow_smem(simt_kernel, kSumBytes + sizeof(float) * kStages * kStageFloats));
     simt_kernel<<<grid, 256, smem, s>>>(P);
     ASD_CUDA_TRY(cudaGetLastError());
     return ASD_OK;

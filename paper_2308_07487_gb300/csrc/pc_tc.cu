@@ -49,7 +49,7 @@ static int configure_once(asd_corr_plan *p, size_t cap, size_t stage_bytes)
 
 int tc_configure(asd_corr_plan *p)
 {
-    const size_t cap = 232448 - 1024 /*alignment slack*/ - 1024 /*barriers*/;
+    const size_t cap = kMaxSmem - 1024 /*alignment slack*/ - 1024 /*barriers*/;
     // (a CTA pair's stage holds this CTA's half of the B columns)
     const size_t stage_bytes = (size_t)p->n_planes * (kBM + p->BN / p->CG) * p->swizzle_bytes;
     int st = configure_once(p, cap, stage_bytes);

@@ -2067,7 +2067,7 @@ int launch_one(const LaunchArgs &a, size_t smem, int sm_count, cudaStream_t s)
 {
     auto k = pc_tc_kernel<FORM, BN, SWB, EW, CG>;
     constexpr int kThreads = tc_threads(BN, EW);
-    ASD_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    ASD_CUDA_TRY(allow_smem(k, kMaxSmem));
     if constexpr (CG == 1) {
         // persistent: one CTA per SM, no more CTAs than work items
         const int grid = (int)(a.total_tiles < sm_count ? a.total_tiles : sm_count);

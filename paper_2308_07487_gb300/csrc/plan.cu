@@ -933,7 +933,7 @@ int asd_pair_corr_batched(asd_corr_plan *const *plans, const float *const *trajs
     uint32_t vb = 0;
     {
         size_t stage_bytes = (size_t)p0->n_planes * (kBM + p0->BN) * p0->swizzle_bytes;
-        const size_t cap = 232448 - 2048;
+        const size_t cap = kMaxSmem - 2048;
         auto region = [&](int k) { return tc_var_bytes(plans[k]->NW, plans[k]->n_bins, nlut[k], p0->EW); };
         auto largest = [&]() {
             uint32_t m = 0;

@@ -164,8 +164,7 @@ int launch_nudft(const float *W, int ldw, int M, const float *X, int64_t K, int6
 {
     constexpr int TN = 256 * U * U / TM;
     constexpr size_t smem = sizeof(float) * kStages * kTS * (TM + TN);
-    ASD_CUDA_TRY(cudaFuncSetAttribute(nudft_kernel<TM, U>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)smem));
+    ASD_CUDA_TRY(allow_smem(nudft_kernel<TM, U>, smem));
     dim3 g((unsigned)((K + TN - 1) / TN), (unsigned)((M + TM - 1) / TM),
            (unsigned)((N + kSlice - 1) / kSlice));
     nudft_kernel<TM, U><<<g, 256, smem, s>>>(W, ldw, M, X, K, N, x16, Fb);

@@ -69,8 +69,7 @@ int asd_sq_omega(const double *S, int n_t, int n_q, double dt, int window, doubl
     ASD_CHECK_ARG(window != 2 || width > 0.0, "Gaussian window needs width > 0");
     const size_t smem = 2 * sizeof(double) * (size_t)n_t;   // 96 KB at most
     if (smem > 48 * 1024)
-        ASD_CUDA_TRY(cudaFuncSetAttribute(sq_omega_kernel,
-                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        ASD_CUDA_TRY(allow_smem(sq_omega_kernel, 2 * sizeof(double) * kMaxNt));
     sq_omega_kernel<<<n_w, 128, smem, (cudaStream_t)stream>>>(S, n_t, n_q, dt, window, width, omega,
                                                               Sqw);
     ASD_CUDA_TRY(cudaGetLastError());
