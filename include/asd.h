@@ -143,7 +143,11 @@ typedef struct asd_corr_plan asd_corr_plan;
  * or positions, per-site cos/sin(q.r_i) tables), computes the exact ordered-pair
  * count of every bin on the device, allocates the operand workspace (BF16 hi/lo or
  * TF32 copies of the trajectory, zero-padded B operand) and encodes the TMA
- * descriptors.  Synchronises the device.  The plan owns all of it.
+ * descriptors.  Synchronises the device.  The plan owns all of it.  An FP32 plan holds
+ * a second copy of the whole trajectory, 4 * S*3F * (N rounded up to a multiple of
+ * four) bytes (2 GB for 64^3 sites and 639 frames), where the device has room for it;
+ * where not, the plan is made without it and _contract reads the trajectory itself:
+ * the same results, more slowly.
  * Errors: ASD_EINVAL (shape/argument), ASD_ENOMEM, ASD_ECUDA, ASD_EUNSUPPORTED
  * (tensor-core form requested on a device without tcgen05).
  */

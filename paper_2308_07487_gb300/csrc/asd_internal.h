@@ -241,8 +241,10 @@ struct asd_corr_plan {
     size_t ws_bytes;
     void *A[2][asd::kMaxCopies];
     void *B[2];
-    float *Af32;              // FP32 form: A operand by K, every value twice [R][ld32]
-    float *Bf32;               // FP32 form: B operand by K [Kb][ld32]
+    float *Af32;               // FP32 form: A operand by K [R][ldk]; null: no room for it, A is
+                               // read from the trajectory
+    float *Bf32;               // FP32 form: B operand by K [Kb][ldk]
+    int64_t ldk;               // sites rounded up to whole 16-byte words, or lines
     int64_t ld32;              // sites rounded up to whole tiles
     float *meanB;              // [N][3] centring means
     // geometry (device)

@@ -20,6 +20,9 @@
 // bins only 58, K = 6144 bins only 60); the steps: operands by K with cp.async and packed FMAs
 // 28.1 (scalar FMAs 29.4; A stored twice per value to save packing 31.6), weights by q in the
 // phase sums (whole lines instead of 16 per load) 24.6, 16 k per stage instead of 8 22.1.
+// A plan without room for its copy of the trajectory by K (DIRECT) loads A from the trajectory
+// row at the K-offset s*3F + 3t, four bytes at a time into the same stages, so with the same
+// sums in the same order: 31.7 ms.
 #include "asd_internal.h"
 #include "geom.cuh"
 
@@ -32,9 +35,10 @@ constexpr int kStageFloats = TK * (TM + TN);   // A, B
 constexpr size_t kSumBytes = 48 * 1024;        // most that the bin and phase sums take
 
 struct SimtParams {
-    const float *A;   // [S*F3][ld]: the trajectory by K
+    const float *A;   // [S*F3][ld]: the trajectory by K (DIRECT: the trajectory [N][R])
     const float *B;   // [S*Kseg][ld]
-    int64_t ld;       // sites, padded to whole tiles
+    int64_t ld;       // sites, padded to whole 16-byte words
+    int64_t R;        // trajectory row length S*F3
     int F3;
     int K3;           // 3*T0
     int Kseg;         // B segment per sample
@@ -66,6 +70,7 @@ __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c)
 }
 
 // (two CTAs per SM: at most 128 registers a thread)
+template <bool DIRECT>
 __global__ void __launch_bounds__(256, 2) simt_kernel(const __grid_constant__ SimtParams P)
 {
     // pipeline stages, then [n_bins] and [n_q][q_parts] FP64, then [8][n_bins] FP32
@@ -91,31 +96,47 @@ __global__ void __launch_bounds__(256, 2) simt_kernel(const __grid_constant__ Si
 
     const int steps_per_seg = P.Kseg / TK;
     const int n_steps = P.S * steps_per_seg;
-    // a stage: 8 k of 128 sites, A as float2 (512 16-byte words: two per thread), B 256.
-    // Rows past the range and k past 3*T0 read as zeros.
+    // a stage: 16 k of 128 sites of each operand, [k][site] (512 16-byte words each, two per
+    // thread, always the same four sites of it).  Rows past the range, columns past the last
+    // site and k past 3*T0 read as zeros.
+    const int four = (tid & 31) * 4;
+    const uint32_t b_bytes = 4u * min(4, max(0, P.N - n0 - four));
+    const int b_col = n0 + (b_bytes ? four : 0);   // (a column that exists where none is read)
     int ls = 0, lk = 0;   // sample and k of the next stage to load
     auto load = [&](int st) {
         if (st < n_steps) {
             float *buf = dyn + (st % kStages) * kStageFloats;
             const uint32_t da = (uint32_t)__cvta_generic_to_shared(buf);
-            const float *A = P.A + ((int64_t)ls * P.F3 + 3 * t + lk) * P.ld + m0;
+            if (DIRECT) {
+                const int k = tid & 15, r0 = tid >> 4;
+                const float *A = P.A + (int64_t)(m0 + r0) * P.R + (int64_t)ls * P.F3 + 3 * t + lk + k;
 #pragma unroll
-            for (int u = 0; u < TK / 8; ++u) {
-                const int e = tid + 256 * u, k = e >> 5, r = (e & 31) * 4;   // four sites
-                const int left = lk + k < P.K3 ? min(4, max(0, P.row_end - m0 - r)) : 0;
-                const float *src = left ? A + k * P.ld + r : P.A;
-                const uint32_t dst = da + (uint32_t)(k * TM + r) * 4;
-                if (P.a16) {
-                    cp_async16(dst, src, 4u * left);
-                } else {
-                    for (int q = 0; q < 4; ++q) cp_async4(dst + 4 * q, left > q ? src + q : P.A, left > q ? 4u : 0u);
+                for (int u = 0; u < TM / 16; ++u) {
+                    const bool ok = lk + k < P.K3 && m0 + r0 + 16 * u < P.row_end;
+                    cp_async4(da + (uint32_t)(k * TM + r0 + 16 * u) * 4,
+                              ok ? A + (int64_t)(16 * u) * P.R : P.A, ok ? 4u : 0u);
+                }
+            } else {
+                const float *A = P.A + ((int64_t)ls * P.F3 + 3 * t + lk) * P.ld + m0 + four;
+#pragma unroll
+                for (int u = 0; u < TK / 8; ++u) {
+                    const int k = (tid >> 5) + 8 * u;
+                    const int left = lk + k < P.K3 ? min(4, max(0, P.row_end - m0 - four)) : 0;
+                    const float *src = left ? A + k * P.ld : P.A;
+                    const uint32_t dst = da + (uint32_t)(k * TM + four) * 4;
+                    if (P.a16) {
+                        cp_async16(dst, src, 4u * left);
+                    } else {
+                        for (int q = 0; q < 4; ++q)
+                            cp_async4(dst + 4 * q, left > q ? src + q : P.A, left > q ? 4u : 0u);
+                    }
                 }
             }
-            const float *B = P.B + ((int64_t)ls * P.Kseg + lk) * P.ld + n0;
+            const float *B = P.B + ((int64_t)ls * P.Kseg + lk) * P.ld + b_col;
 #pragma unroll
             for (int u = 0; u < TK / 8; ++u) {
-                const int e = tid + 256 * u, k = e >> 5, c = (e & 31) * 4;
-                cp_async16(da + (uint32_t)(TK * TM + k * TN + c) * 4, B + k * P.ld + c, 16u);
+                const int k = (tid >> 5) + 8 * u;
+                cp_async16(da + (uint32_t)(TK * TM + k * TN + four) * 4, B + k * P.ld, b_bytes);
             }
             lk += TK;
             if (lk == P.Kseg) {
@@ -266,9 +287,10 @@ int launch_simt(asd_corr_plan *p, int64_t row_begin, int64_t row_end, int t_begi
                 double *C_sum, double *Sq_sum, cudaStream_t s)
 {
     SimtParams P{};
-    P.A = p->Af32;
+    P.A = p->Af32 ? p->Af32 : p->prepared_traj;
+    P.R = p->R;
     P.B = p->Bf32;
-    P.ld = p->ld32;
+    P.ld = p->ldk;
     P.a16 = (row_begin & 3) == 0;
     P.F3 = 3 * p->F;
     P.K3 = 3 * p->T0;
@@ -312,8 +334,9 @@ int launch_simt(asd_corr_plan *p, int64_t row_begin, int64_t row_end, int t_begi
     P.warp_bins = !p->d.deterministic && smem + sizeof(float) * 8 * p->n_bins <= kSumBytes;
     if (P.warp_bins) smem += sizeof(float) * 8 * p->n_bins;
     smem += sizeof(float) * kStages * kStageFloats;
-    ASD_CUDA_TRY(allow_smem(simt_kernel, kSumBytes + sizeof(float) * kStages * kStageFloats));
-    simt_kernel<<<grid, 256, smem, s>>>(P);
+    auto k = p->Af32 ? simt_kernel<false> : simt_kernel<true>;
+    ASD_CUDA_TRY(allow_smem(k, kSumBytes + sizeof(float) * kStages * kStageFloats));
+    k<<<grid, 256, smem, s>>>(P);
     ASD_CUDA_TRY(cudaGetLastError());
     return ASD_OK;
 }

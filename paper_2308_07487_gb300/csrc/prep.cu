@@ -252,7 +252,7 @@ int launch_prep(asd_corr_plan *p, const float *traj, int64_t row_begin, int64_t 
         Prep32Args a{};
         a.traj = traj;
         a.N = p->N;
-        a.ld = p->ld32;
+        a.ld = p->ldk;
         a.R = p->R;
         a.row_begin = row_begin;
         a.row_end = row_end;
@@ -265,9 +265,9 @@ int launch_prep(asd_corr_plan *p, const float *traj, int64_t row_begin, int64_t 
         a.A = p->Af32;
         a.B = p->Bf32;
         a.tiles_a_k = (p->R + 31) / 32;
-        a.tiles_a = a.tiles_a_k * ((row_end - row_begin + 31) / 32);
+        a.tiles_a = p->Af32 ? a.tiles_a_k * ((row_end - row_begin + 31) / 32) : 0;
         a.tiles_b_k = (p->Kb + 31) / 32;
-        a.tiles = a.tiles_a + a.tiles_b_k * (p->ld32 / 32);
+        a.tiles = a.tiles_a + a.tiles_b_k * ((p->ldk + 31) / 32);
         const int64_t blocks = a.tiles < (1 << 20) ? a.tiles : 1 << 20;
         prep32_kernel<<<(unsigned)blocks, 256, 0, s>>>(a);
         ASD_CUDA_TRY(cudaGetLastError());
