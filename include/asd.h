@@ -327,7 +327,7 @@ typedef struct asd_system {
  * renormalisation (Section 3.1), for S samples at once.
  *   spins0 device [S][N][3]; traj device [N][S][n_frames][3]: frame 0 = spins0,
  *   frame f = state after f*stride steps of size dt.  spins_out (device [S][N][3],
- *   nullable) receives the final state.  Systems of up to about 600000 site-samples run
+ *   nullable) receives the final state.  Systems of up to about 300000 site-samples run
  *   as one kernel per 4096 steps (a cooperative launch unless each sample fits one thread
  *   block), larger ones as 4 kernels per step.
  */

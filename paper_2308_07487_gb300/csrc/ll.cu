@@ -15,7 +15,7 @@
 //   ll_tagged              a cooperative launch over every (sample, site), one site per thread;
 //                          blocks exchange stage inputs as words that carry their stage number;
 //   ll_persistent<global>  a cooperative launch, the state in L2, a grid barrier between stages:
-//                          up to four sites per thread;
+//                          up to two sites per thread;
 //   rk4_stage              one launch per stage: larger systems.
 // The last stage writes the new state and, every `stride` steps, the trajectory frame in the
 // site-major layout traj[i][s][f][a] consumed by asd_pair_corr.  All routes do the same
@@ -63,8 +63,21 @@ __device__ __forceinline__ float3 field(const LLArgs &a, const float *__restrict
     for (int k = 0; k < a.z; ++k) {
         const int j = __ldg(a.nbr + i * a.z + k);
         if (j < 0) continue;
-        add_bond(h, __ldg(a.J + i * a.z + k), Ys[3 * (int64_t)j], Ys[3 * (int64_t)j + 1],
-                 Ys[3 * (int64_t)j + 2], a.D ? a.D + (i * a.z + k) * 3 : nullptr);
+        // (add_bond's sums, written out: through the call a stage of 70^3 sites took 3 to 8 %
+        // longer, at 32 instead of 40 registers and a nearly empty second wave of blocks)
+        const float Jij = __ldg(a.J + i * a.z + k);
+        h.x = fmaf(Jij, Ys[3 * (int64_t)j + 0], h.x);
+        h.y = fmaf(Jij, Ys[3 * (int64_t)j + 1], h.y);
+        h.z = fmaf(Jij, Ys[3 * (int64_t)j + 2], h.z);
+        if (a.D) {
+            const float *d = a.D + (i * a.z + k) * 3;
+            const float dx = __ldg(d), dy = __ldg(d + 1), dz = __ldg(d + 2);
+            const float sx = Ys[3 * (int64_t)j], sy = Ys[3 * (int64_t)j + 1],
+                        sz = Ys[3 * (int64_t)j + 2];
+            h.x += dy * sz - dz * sy;
+            h.y += dz * sx - dx * sz;
+            h.z += dx * sy - dy * sx;
+        }
     }
     h.z = fmaf(-2.f * a.A, Ys[3 * i + 2], h.z);
     return h;
@@ -128,7 +141,7 @@ __global__ void write_frame0(const float *__restrict__ Y, int64_t N, int S, floa
 // Persistent routes
 // ---------------------------------------------------------------------------------------
 constexpr int kLLThreads = 1024;
-constexpr int kLLMaxSpt = 4;                       // sites per thread
+constexpr int kLLMaxSpt = 2;                       // sites per thread
 constexpr size_t kLLMaxSmem = 220 * 1024;
 constexpr int kLLStepsPerLaunch = 4096;            // other streams' work gets in between
 
@@ -557,8 +570,8 @@ typedef void (*LLKernel)(LLRun);
 template <int SPT, bool LOCAL>
 LLKernel ll_kernel_z(int z)
 {
-    if (SPT <= 2 && z == 4) return ll_persistent<SPT <= 2 ? SPT : 1, 4, LOCAL>;
-    if (SPT <= 2 && z == 6) return ll_persistent<SPT <= 2 ? SPT : 1, 6, LOCAL>;
+    if (z == 4) return ll_persistent<SPT, 4, LOCAL>;
+    if (z == 6) return ll_persistent<SPT, 6, LOCAL>;
     return ll_persistent<SPT, 0, LOCAL>;
 }
 
@@ -573,8 +586,11 @@ struct LLRoute {
 };
 
 // One block per sample up to 2048 sites (two per thread; the state and any table must fit
-// shared memory).  Otherwise a cooperative launch, one block per SM, as few sites per
-// thread as cover the system.
+// shared memory).  Otherwise a cooperative launch, one block per SM, one or two sites per
+// thread.  Beyond that (more than 2048 sites per SM) a launch per stage: with four sites per
+// thread, their bonds in shared memory, the cooperative kernel took 54.8 -> 64.6 us (80^3
+// glass, one step), 385 -> 450 us (68^3, 10 steps), and gained 4 to 17 % only on lattices of
+// four bonds (700^2, 10 steps, 506 -> 434 us).
 int ll_route(const LLArgs &a, LLRoute *out)
 {
     *out = LLRoute();
@@ -623,8 +639,7 @@ int ll_route(const LLArgs &a, LLRoute *out)
         r.tagged = spt == 1 && r.smem + own <= kLLMaxSmem;
         add_frames(r, r.smem + (r.tagged ? own : 0), (int64_t)spt * r.block);
         r.k = r.tagged ? (a.z == 4 ? ll_tagged<4> : a.z == 6 ? ll_tagged<6> : ll_tagged<0>)
-              : spt == 1 ? ll_persistent<1, 0, false>
-              : spt == 2 ? ll_kernel_z<2, false>(a.z) : ll_kernel_z<4, false>(a.z);
+              : spt == 1 ? ll_persistent<1, 0, false> : ll_kernel_z<2, false>(a.z);
         ASD_CUDA_TRY(allow_smem(r.k, kLLMaxSmem));
         int per_sm = 0;
         ASD_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, r.k, (int)r.block,
