@@ -10,8 +10,8 @@
 // notes its RK4 evolution is not norm preserving.
 //
 // A stage needs every neighbour's previous stage.  Routes, by size (ll_run):
-//   ll_persistent<LOCAL>   one block per sample, the state in shared memory, a block barrier
-//                          between stages: samples of up to 2048 sites;
+//   ll_persistent<LOCAL>   one block per sample, or per several small ones, the state in shared
+//                          memory, a block barrier between stages: samples of up to 2048 sites;
 //   ll_tagged              a cooperative launch over every (sample, site), one site per thread;
 //                          blocks exchange stage inputs as words that carry their stage number;
 //   ll_persistent<global>  a cooperative launch, the state in L2, a grid barrier between stages:
@@ -142,6 +142,7 @@ __global__ void write_frame0(const float *__restrict__ Y, int64_t N, int S, floa
 // ---------------------------------------------------------------------------------------
 constexpr int kLLThreads = 1024;
 constexpr int kLLMaxSpt = 2;                       // sites per thread
+constexpr int64_t kLLPackSites = 256;              // sites of small samples per block
 constexpr size_t kLLMaxSmem = 220 * 1024;
 constexpr int kLLStepsPerLaunch = 4096;            // other streams' work gets in between
 
@@ -151,6 +152,7 @@ struct LLRun {
     float *out;          // [S][N][3] state after the last step, or null
     float4 *Y, *T1, *T2; // global route: state and stage inputs [S][N]
     int n_buf;           // ll_tagged: stage inputs from Y on, 2 .. kLLMaxBufs
+    int per_block;       // samples per block (PACK)
     unsigned *bar;       // cooperative routes: grid barrier count (zero at launch)
     float *traj;
     int F;
@@ -175,7 +177,7 @@ constexpr int kLLFramePitch = 3 * kLLFrames + 1;   // words per site (odd: no ba
 // which the barrier about 2); frames stored by each site as they come instead of gathered:
 // 130 us and 3.78 ms.  36^2 sites and two samples, 90 steps: 1.58 -> 0.53 ms, though only
 // two blocks run.
-template <int SPT, int Z, bool LOCAL>
+template <int SPT, int Z, bool LOCAL, bool PACK = false>
 __global__ void __launch_bounds__(kLLThreads, 1) ll_persistent(const __grid_constant__ LLRun r)
 {
     extern __shared__ __align__(16) uint8_t ll_smem[];
@@ -183,17 +185,17 @@ __global__ void __launch_bounds__(kLLThreads, 1) ll_persistent(const __grid_cons
     const LLArgs &a = r.a;
     const int N = (int)a.N, nt = blockDim.x, tid = threadIdx.x;
     const int64_t n = (int64_t)N * a.S;
-    // LOCAL: block = sample, site = tid + k nt.  Else sites of the flattened (sample, site)
-    // list in contiguous runs of SPT nt per block.
-    const int64_t g0 = LOCAL ? (int64_t)blockIdx.x * N : (int64_t)blockIdx.x * SPT * nt;
+    // contiguous runs of the flattened (sample, site) list per block: LOCAL a sample (PACK:
+    // per_block of them), else SPT nt sites.  Slot = site index within the block, tid + k nt.
+    const int slots = LOCAL ? (PACK ? r.per_block * N : N) : SPT * nt;
+    const int64_t g0 = (int64_t)blockIdx.x * slots;
     // state arrays indexed by the flattened site minus `base`
     const int64_t base = LOCAL ? g0 : 0;
     float4 *Y = LOCAL ? reinterpret_cast<float4 *>(ll_smem) : r.Y;
-    float4 *T1 = LOCAL ? Y + N : r.T1;
-    float4 *T2 = LOCAL ? T1 + N : r.T2;
-    // bonds in shared memory: [k][slot], slot = site index within the block
-    int *sm_nbr = reinterpret_cast<int *>(ll_smem + (LOCAL ? (size_t)48 * N : 0));
-    const int slots = LOCAL ? N : SPT * nt;
+    float4 *T1 = LOCAL ? Y + slots : r.T1;
+    float4 *T2 = LOCAL ? T1 + slots : r.T2;
+    // bonds in shared memory: [k][slot]
+    int *sm_nbr = reinterpret_cast<int *>(ll_smem + (LOCAL ? (size_t)48 * slots : 0));
     float *sm_J = reinterpret_cast<float *>(sm_nbr + (kReg ? 0 : (size_t)a.z * slots));
     float *sm_frames = sm_J + (kReg ? 0 : (size_t)a.z * slots);
 
@@ -209,9 +211,9 @@ __global__ void __launch_bounds__(kLLThreads, 1) ll_persistent(const __grid_cons
     for (int u = 0; u < SPT; ++u) {
         const int slot = u * nt + tid;
         const int64_t g = g0 + slot;
-        on[u] = LOCAL ? slot < N : g < n;
+        on[u] = LOCAL && !PACK ? slot < N : slot < slots && g < n;
         const int64_t gc = on[u] ? g : g0;
-        const int s = LOCAL ? (int)blockIdx.x : (int)(gc / N);
+        const int s = LOCAL && !PACK ? (int)blockIdx.x : (int)(gc / N);
         site[u] = (int)(gc - (int64_t)s * N);
         const int off = (int)((int64_t)s * N - base);   // the sample's first index
         own[u] = (int)(gc - base);
@@ -248,11 +250,12 @@ __global__ void __launch_bounds__(kLLThreads, 1) ll_persistent(const __grid_cons
     int64_t f_held = r.step0 / r.stride + 1;    // first frame held
     auto put_frames = [&]() {
         __syncthreads();   // every site's frames are in
-        const int words = 3 * n_held, left = LOCAL ? N : (int)min((int64_t)slots, n - g0);
+        const int words = 3 * n_held,
+                  left = LOCAL && !PACK ? N : (int)min((int64_t)slots, n - g0);
         for (int e = tid; e < left * words; e += nt) {
             const int slot = e / words, c = e - slot * words;
             const int64_t g = g0 + slot;
-            const int64_t s = LOCAL ? blockIdx.x : g / N, i = g - s * N;
+            const int64_t s = LOCAL && !PACK ? blockIdx.x : g / N, i = g - s * N;
             r.traj[((i * a.S + s) * r.F + f_held) * 3 + c] = sm_frames[slot * kLLFramePitch + c];
         }
         f_held += n_held;
@@ -582,11 +585,15 @@ struct LLRoute {
     bool local = false, tagged = false;
     unsigned grid = 0, block = 0;
     size_t smem = 0;
+    int per_block = 1;   // local: samples per block
     bool stage_frames = false;
 };
 
 // One block per sample up to 2048 sites (two per thread; the state and any table must fit
-// shared memory).  Otherwise a cooperative launch, one block per SM, one or two sites per
+// shared memory; samples of up to 48 sites share blocks where there are more than the
+// device holds at once (32 blocks per SM): 300000 samples of one site, one step, 213 us in a warp
+// each, 12.4 shared, 37 by a launch per stage; of 4 sites 262, 45 and 77; of 64 sites 50 us for
+// 20000 in blocks of their own, 57 shared).  Otherwise a cooperative launch, one block per SM, one or two sites per
 // thread.  Beyond that (more than 2048 sites per SM) a launch per stage: with four sites per
 // thread, their bonds in shared memory, the cooperative kernel took 54.8 -> 64.6 us (80^3
 // glass, one step), 385 -> 450 us (68^3, 10 steps), and gained 4 to 17 % only on lattices of
@@ -617,9 +624,17 @@ int ll_route(const LLArgs &a, LLRoute *out)
         if (smem <= kLLMaxSmem) {
             r.local = true;
             r.k = spt == 1 ? ll_kernel_z<1, true>(a.z) : ll_kernel_z<2, true>(a.z);
-            r.grid = (unsigned)a.S;
-            r.block = (unsigned)(((a.N + spt - 1) / spt + 31) / 32 * 32);
-            add_frames(r, smem, a.N);
+            // more samples than blocks fit the device at once (32 per SM): several per block
+            if (a.S > 32 * sms && a.N <= 48) {
+                r.per_block = (int)(kLLPackSites / a.N);
+                r.k = a.z == 4   ? ll_persistent<1, 4, true, true>
+                      : a.z == 6 ? ll_persistent<1, 6, true, true>
+                                 : ll_persistent<1, 0, true, true>;
+            }
+            const int64_t slots = r.per_block * a.N;
+            r.grid = (unsigned)((a.S + r.per_block - 1) / r.per_block);
+            r.block = (unsigned)(((slots + spt - 1) / spt + 31) / 32 * 32);
+            add_frames(r, (size_t)48 * slots + bonds(spt, slots), slots);
             ASD_CUDA_TRY(allow_smem(r.k, kLLMaxSmem));
             *out = r;
             return ASD_OK;
@@ -678,6 +693,7 @@ int ll_run(const LLArgs &a, const LLRoute &rt, const float *spins0, float dt, in
         r.stride = stride;
         r.dt = dt;
         r.stage_frames = rt.stage_frames;
+        r.per_block = rt.per_block;
         r.err = device_error_word();
         if (!r.err) return ASD_ECUDA;
         const float *in = spins0;
