@@ -162,6 +162,7 @@ struct LLRun {
     int stage_frames;    // 1: frames go out through shared memory, kLLFrames at a time
     int *err;
 };
+constexpr int kLLGroup = 4;                         // bonds loaded together (Z = 0)
 constexpr int kLLMaxBufs = 9;                       // stage inputs of ll_tagged
 constexpr int kLLFrames = 4;
 constexpr int kLLFramePitch = 3 * kLLFrames + 1;   // words per site (odd: no bank conflicts)
@@ -292,13 +293,31 @@ __global__ void __launch_bounds__(kLLThreads, 1) ll_persistent(const __grid_cons
                     add_bond(h, kReg ? Jr[kReg ? k : 0] : sm_J[k * slots + slot], sj[k].x,
                              sj[k].y, sj[k].z,
                              a.D ? a.D + ((int64_t)site[u] * Z + k) * 3 : nullptr);
-        } else {
+        } else if (LOCAL) {
             for (int k = 0; k < a.z; ++k) {
                 const int j = sm_nbr[k * slots + slot];
                 if (j < 0) continue;
                 const float4 sj = V[j];
                 add_bond(h, sm_J[k * slots + slot], sj.x, sj.y, sj.z,
                          a.D ? a.D + ((int64_t)site[u] * a.z + k) * 3 : nullptr);
+            }
+        } else {
+            // from L2: a group's loads in flight together (one after the other, the 26 bonds of a
+            // stage took 9 us, more than a launch per stage: 12^3 sites, 40 stages, 379 -> 204 us;
+            // from shared memory, above, groups gain nothing and cost 10 % with DM vectors)
+            for (int k0 = 0; k0 < a.z; k0 += kLLGroup) {
+                float4 sj[kLLGroup];
+                int j[kLLGroup];
+#pragma unroll
+                for (int q = 0; q < kLLGroup; ++q) {
+                    j[q] = k0 + q < a.z ? sm_nbr[(k0 + q) * slots + slot] : -1;
+                    sj[q] = V[j[q] < 0 ? own[u] : j[q]];
+                }
+#pragma unroll
+                for (int q = 0; q < kLLGroup; ++q)
+                    if (j[q] >= 0)
+                        add_bond(h, sm_J[(k0 + q) * slots + slot], sj[q].x, sj[q].y, sj[q].z,
+                                 a.D ? a.D + ((int64_t)site[u] * a.z + k0 + q) * 3 : nullptr);
             }
         }
         h.z = fmaf(-2.f * a.A, x[u].z, h.z);
@@ -504,12 +523,24 @@ __global__ void __launch_bounds__(kLLThreads, 1) ll_tagged(const __grid_constant
                     add_bond(h, Jr[k], sj[k].x, sj[k].y, sj[k].z,
                              a.D ? a.D + ((int64_t)site * Z + k) * 3 : nullptr);
         } else {
-            for (int k = 0; k < a.z; ++k) {
-                const int j = sm_nbr[k * nt + tid];
-                if (j == -1) continue;
-                const float4 sj = j >= 0 ? V[j] : wait_tagged(G - (j + 2), g);
-                add_bond(h, sm_J[k * nt + tid], sj.x, sj.y, sj.z,
-                         a.D ? a.D + ((int64_t)site * a.z + k) * 3 : nullptr);
+            for (int k0 = 0; k0 < a.z; k0 += kLLGroup) {   // (as above, a group at a time)
+                float4 sj[kLLGroup];
+                int j[kLLGroup];
+#pragma unroll
+                for (int q = 0; q < kLLGroup; ++q) {
+                    j[q] = k0 + q < a.z ? sm_nbr[(k0 + q) * nt + tid] : -1;
+                    if (j[q] >= -1) sj[q] = V[j[q] < 0 ? tid : j[q]];
+                    else sj[q] = ld_tagged(G - (j[q] + 2));
+                }
+#pragma unroll
+                for (int q = 0; q < kLLGroup; ++q)
+                    if (j[q] < -1 && __float_as_int(sj[q].w) != g)
+                        sj[q] = wait_tagged(G - (j[q] + 2), g);
+#pragma unroll
+                for (int q = 0; q < kLLGroup; ++q)
+                    if (j[q] != -1)
+                        add_bond(h, sm_J[(k0 + q) * nt + tid], sj[q].x, sj[q].y, sj[q].z,
+                                 a.D ? a.D + ((int64_t)site * a.z + k0 + q) * 3 : nullptr);
             }
         }
         h.z = fmaf(-2.f * a.A, x.z, h.z);
