@@ -254,7 +254,7 @@ __global__ void mc_color_kernel(MCArgs a, float *__restrict__ spins)
 // ---------------------------------------------------------------------------------------
 constexpr int kMcMaxColors = 16;
 constexpr int kMcSweepsPerLaunch = 4096;   // other streams' work gets in between
-constexpr int kMcLocalSites = 4096;
+constexpr int kMcLocalSites = 2048, kMcLocalMost = 4096;
 
 struct MCRun {
     MCArgs a;                         // (per-colour fields unused)
@@ -449,16 +449,42 @@ struct MCRoute {
     size_t smem = 0;
 };
 
-// A block per sample up to kMcLocalSites sites (adaptive runs of several samples share one
-// cone, so they take the grid route); else the grid route, at most one block per SM.
-int mc_route(const MCArgs &a, const int64_t *off, int n_colors, int adapt, int sms, MCRoute *out)
+// Where the sweeps run: a block per sample (local), a cooperative launch over all samples (grid,
+// at most one block per SM), or a launch per colour.  Adaptive runs of several samples share
+// one cone, so they take the grid.
+//
+// One block is soon slower than the device, so local up to kMcLocalSites sites: 64^2, one chain,
+// one sweep 21.7 us in a block, 13.4 by the grid, 17.1 by a launch per colour, ten sweeps 106, 69
+// and 121; 44^2 15.7, 13.3 and 17.4, 56.6, 69.2 and 129; 16^3 with 26 bonds and DM vectors, ten
+// sweeps, 1510, 744 and 965.  Twice as many where the grid's threads would each have several
+// sites of a colour (but not many, where the grid's better balance pays): 152 chains of 64^2,
+// ten sweeps, 110, 162 and 274.  Not local: one sweep of more sites than the device takes at
+// once (300000 chains of 64 sites 392, 280 and 358), and samples of less than a warp per
+// colour, more of them than there are blocks (300000 of one site, ten sweeps, 1147, 97 and 121).
+//
+// A launch per colour has more threads and so more loads in flight, which is what many bonds
+// need on more sites than the grid has threads: 26 bonds, 400 chains of 16^3, one sweep, 285 us
+// by the grid, 247 by launches; 1000 chains, ten sweeps, 5080 local, 4730; 12 bonds with DM
+// vectors, 1000 chains, ten sweeps, 4930 local, 4650 and 4330.  And one pass over one colour has
+// nothing to keep between launches.
+int mc_route(const MCArgs &a, const int64_t *off, int n_colors, int n_sweeps, int adapt, int sms,
+             MCRoute *out)
 {
     *out = MCRoute();
     if (n_colors > kMcMaxColors || a.proposal == ASD_LEARNED) return ASD_OK;
-    int64_t widest = 0;
-    for (int c = 0; c < n_colors; ++c) widest = std::max(widest, off[c + 1] - off[c]);
+    int64_t widest = 0, passes = 0;
+    for (int c = 0; c < n_colors; ++c) {
+        widest = std::max(widest, off[c + 1] - off[c]);
+        if (off[c + 1] > off[c]) passes += n_sweeps;
+    }
+    const int64_t full = 1024 * (int64_t)sms, load = widest * a.S;
+    const bool filled = load > full / 4 * 3;
+    if (filled && (a.z > 8 || (a.D && a.z > 6))) return ASD_OK;
     MCRoute r;
-    if (a.N <= kMcLocalSites && (!adapt || a.S == 1)) {
+    const bool local = (a.N <= kMcLocalSites ||
+                        (a.N <= kMcLocalMost && filled && load <= 4 * full)) &&
+                       !(filled && n_sweeps == 1) && !(widest < 32 && a.S > 32 * sms);
+    if (local && (!adapt || a.S == 1)) {
         r.local = true;
         r.k = a.z == 4   ? mc_persistent<4, true>
               : a.z == 6 ? mc_persistent<6, true>
@@ -466,10 +492,11 @@ int mc_route(const MCArgs &a, const int64_t *off, int n_colors, int adapt, int s
         r.grid = (unsigned)a.S;
         r.block = (unsigned)std::min<int64_t>(1024, (widest + 31) / 32 * 32);
         r.smem = sizeof(float4) * (size_t)a.N;
-        ASD_CUDA_TRY(allow_smem(r.k, sizeof(float4) * kMcLocalSites));
+        ASD_CUDA_TRY(allow_smem(r.k, sizeof(float4) * kMcLocalMost));
         *out = r;
         return ASD_OK;
     }
+    if (passes <= 1) return ASD_OK;
     int dev = 0, coop = 0, per_sm = 0;
     ASD_CUDA_TRY(cudaGetDevice(&dev));
     ASD_CUDA_TRY(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
@@ -760,7 +787,7 @@ extern "C" int asd_thermalize(const asd_system *sys, int n_samples, float *spins
         a.stats = cnt;
         a.net = view;
         MCRoute rt;
-        if ((rc = mc_route(a, sys->color_offsets, sys->n_colors,
+        if ((rc = mc_route(a, sys->color_offsets, sys->n_colors, n_sweeps,
                            adapt && proposal == ASD_METROPOLIS, sms, &rt)))
             break;
         if (rt.k) {
