@@ -1372,7 +1372,7 @@ __global__ void __launch_bounds__(tc_threads(BN, EW), 1) pc_tc_kernel(const __gr
             __syncwarp();
             if (lane == 0) mbar_arrive(wqempty0 + 8 * qs);
             if (p < 0) break;
-            if (!first) continue;
+            if (!first || probs[p].epi.n_bins == 0) continue;   // (phase sums need no geometry)
             const uint32_t gb = item & 1;
             ok = mbar_wait(gempty0 + 8 * gb, ((item >> 1) & 1) ^ 1u, args.err, DEV_TIMEOUT_EPI);
             if (!__all_sync(0xffffffffu, ok)) break;
@@ -1622,7 +1622,7 @@ __global__ void __launch_bounds__(tc_threads(BN, EW), 1) pc_tc_kernel(const __gr
                 float2 cw[32];
 #pragma unroll
                 for (int k = 0; k < 32; ++k)
-                    if (q0 + (k & 16) < n_q) cw[k] = cs[(int64_t)(q0 + k) * ld];
+                    if (q0 + (k & 24) < n_q) cw[k] = cs[(int64_t)(q0 + k) * ld];
                     else cw[k] = make_float2(0.f, 0.f);
                 const int h = q0 & 32;   // second half of the pass
                 if (h == 0) {
@@ -1635,6 +1635,7 @@ __global__ void __launch_bounds__(tc_threads(BN, EW), 1) pc_tc_kernel(const __gr
                 float xs = 0.f, ys = 0.f;   // this lane's q of the 32
 #pragma unroll
                 for (int j = 0; j < 32; j += 8) {
+                    if (q0 + j >= n_q) break;   // (few q-vectors: 8 at a time, not 64)
                     uint32_t u[8], w[8];
                     tmem_ld8(pt + h + j, u);
                     tmem_ld8(pt + kPhaseQ + h + j, w);
@@ -1843,7 +1844,7 @@ __global__ void __launch_bounds__(tc_threads(BN, EW), 1) pc_tc_kernel(const __gr
                 new_t = true;
             }
             if (got && !end) {
-                if (first)
+                if (first && E.n_bins > 0)
                     got = mbar_wait(gfull0 + 8 * (item & 1), (item >> 1) & 1, args.err,
                                     DEV_TIMEOUT_EPI);
                 got = got && mbar_wait(tfull0 + 8 * acc, use & 1, args.err, DEV_TIMEOUT_EPI);
@@ -1852,11 +1853,11 @@ __global__ void __launch_bounds__(tc_threads(BN, EW), 1) pc_tc_kernel(const __gr
             ok = epi_sync_and(got, kEpiThreads);
             if (!ok || end) break;
             tc_after();
-            if (first) {
-                if (new_t) {
-                    flush_acc(cur_p, cur_t);
-                    cur_t = t;
-                }
+            if (first && new_t) {
+                flush_acc(cur_p, cur_t);
+                cur_t = t;
+            }
+            if (first && E.n_bins > 0) {
                 const uint32_t gb = item & 1;
                 colgeo = reinterpret_cast<const float *>(epi + EL.geo) + gb * 3 * BN;
                 tw = reinterpret_cast<const TileWindow *>(epi + EL.win)[gb];
@@ -1973,7 +1974,7 @@ __global__ void __launch_bounds__(tc_threads(BN, EW), 1) pc_tc_kernel(const __gr
                 else mbar_arrive(a);
             }
             // the tile's geometry buffer may be filled again
-            if (last && lane == 0) mbar_arrive(gempty0 + 8 * ((item - 1) & 1));
+            if (last && E.n_bins > 0 && lane == 0) mbar_arrive(gempty0 + 8 * ((item - 1) & 1));
             if (last) epi_sync(kEpiThreads);  // all private bins written
             if (bins_on && last) {
                 // private rows this tile may have written: with the branch-free position
