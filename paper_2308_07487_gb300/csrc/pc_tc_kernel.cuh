@@ -592,6 +592,32 @@ struct BinArgs {
 
 enum { BIN_LUT = 0, BIN_THR = 1, BIN_POS = 2 };
 
+// The values of N pairs (of a chunk, from column k0 on) into this thread's private bins (slot >= 0)
+// or the shared fallback bins (slot -1 - bin), in column order.
+template <int STRIDE, int N>
+__device__ __forceinline__ void add_slots(const uint32_t (&g)[32], int k0, const int (&slot)[N],
+                                          bool row_ok,
+                                          float *__restrict__ myb, void *__restrict__ fbv,
+                                          const BinArgs &ba)
+{
+    const bool det = ba.fscale != 0.0;
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+        // rows past the range: their accumulator rows may come from A rows that were
+        // never prepared, so the value is replaced (a product with 0 would keep a NaN)
+        const float val = row_ok ? __uint_as_float(g[k0 + k]) : 0.f;
+        if (slot[k] < 0) {
+            const int b = -1 - slot[k];
+            if (!ASD_INB(b < ba.NB, BND_FALLBACK, ba.err)) continue;
+            // deterministic mode: fixed-point sums (integer adds in any order)
+            if (det) add_fixed(static_cast<long long *>(fbv) + b, to_fixed(val, ba.fscale));
+            else atomicAdd(static_cast<float *>(fbv) + b, val);
+        } else if (ASD_INB(slot[k] <= ba.trash, BND_PRIV, ba.err)) {
+            myb[slot[k] * STRIDE] += val;
+        }
+    }
+}
+
 // Bin 32 consecutive columns of one accumulator row.  Phase 1 computes the exact bin
 // slot of every pair (loads of geometry and tables only, so the 32 independent chains
 // overlap); phase 2 adds the 32 values into this thread's private bins (its column of
@@ -629,22 +655,7 @@ __device__ __forceinline__ void bin_chunk(const uint32_t (&g)[32], bool row_ok, 
         const int lb = b - ba.blo;
         slot[k] = (unsigned)lb < (unsigned)ba.nwp ? lb : (b < ba.nb ? -1 - b : ba.trash);
     }
-    const bool det = ba.fscale != 0.0;
-#pragma unroll
-    for (int k = 0; k < 32; ++k) {
-        // rows past the range: their accumulator rows may come from A rows that were
-        // never prepared, so the value is replaced (a product with 0 would keep a NaN)
-        const float val = row_ok ? __uint_as_float(g[k]) : 0.f;
-        if (slot[k] < 0) {
-            const int b = -1 - slot[k];
-            if (!ASD_INB(b < ba.NB, BND_FALLBACK, ba.err)) continue;
-            // deterministic mode: fixed-point sums (integer adds in any order)
-            if (det) add_fixed(static_cast<long long *>(fbv) + b, to_fixed(val, ba.fscale));
-            else atomicAdd(static_cast<float *>(fbv) + b, val);
-        } else if (ASD_INB(slot[k] <= ba.trash, BND_PRIV, ba.err)) {
-            myb[slot[k] * STRIDE] += val;
-        }
-    }
+    add_slots<STRIDE>(g, 0, slot, row_ok, myb, fbv, ba);
 }
 
 // ---- branch-free binning: packed FP32 pairs, two columns per instruction ----
@@ -743,13 +754,13 @@ __device__ __forceinline__ void bin2(uint32_t &o0, uint32_t &o1, uint64_t d2, co
 
 // FP32 positions: the squared distance is position_d2's, fma(dz, dz, fma(dy, dy, dx dx))
 // of FP32 differences, for the row at minus (nx, ny, nz) and columns stored by component.
-template <bool EXACT, bool DROP, int STRIDE>
-__device__ __forceinline__ void pos_offsets(uint32_t (&off)[32], uint64_t nx, uint64_t ny,
+template <bool EXACT, bool DROP, int STRIDE, int N>
+__device__ __forceinline__ void pos_offsets(uint32_t (&off)[N], uint64_t nx, uint64_t ny,
                                             uint64_t nz, const float *__restrict__ cg, int BN,
                                             const FastBin &fb)
 {
 #pragma unroll
-    for (int k = 0; k < 32; k += 4) {
+    for (int k = 0; k < N; k += 4) {
         const float4 X = *reinterpret_cast<const float4 *>(cg + k);
         const float4 Y = *reinterpret_cast<const float4 *>(cg + BN + k);
         const float4 Z = *reinterpret_cast<const float4 *>(cg + 2 * BN + k);
@@ -766,6 +777,34 @@ __device__ __forceinline__ void pos_offsets(uint32_t (&off)[32], uint64_t nx, ui
         d = add2(pack2(Z.z, Z.w), nz);
         s = fma2(d, d, s);
         bin2<EXACT, DROP, STRIDE>(off[k + 2], off[k + 3], s, fb);
+    }
+}
+
+// bin_chunk for FP32 positions under the branch-free rule: tiles whose bins do not fit the private
+// window.  24^3 glass in row order, 256 bins of 0.17, K = 192, 16 displacements, split-BF16: 37.2 ms
+// before the binning above took registers from bin_chunk, 38.6 with it, 34.9 here.
+template <int STRIDE>
+__device__ __forceinline__ void pos_chunk(const uint32_t (&g)[32], bool row_ok, float4 rp,
+                                          const float *__restrict__ cg, int BN,
+                                          const float *__restrict__ thr, float *__restrict__ myb,
+                                          void *__restrict__ fbv, const BinArgs ba)
+{
+    const FastBin fb = {pack2(ba.inv_w, ba.inv_w), 0ull, reinterpret_cast<const float2 *>(thr),
+                        ba.nb, 0u - kBinBaseBits, (uint32_t)ba.nb};
+    // (eight columns at a time: the registers of a whole chunk would be taken from the usual
+    // path, 48^3 glass BF16 85.4 -> 86.7 ms; now 86.0)
+#pragma unroll
+    for (int h = 0; h < 32; h += 8) {
+        uint32_t bin[8];
+        pos_offsets<false, true, 1>(bin, pack2(-rp.x, -rp.x), pack2(-rp.y, -rp.y),
+                                    pack2(-rp.z, -rp.z), cg + h, BN, fb);
+        int slot[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const int b = (int)bin[k], lb = b - ba.blo;
+            slot[k] = (unsigned)lb < (unsigned)ba.nwp ? lb : (b < ba.nb ? -1 - b : ba.trash);
+        }
+        add_slots<STRIDE>(g, h, slot, row_ok, myb, fbv, ba);
     }
 }
 
@@ -1949,6 +1988,8 @@ __global__ void __launch_bounds__(tc_threads(BN, EW), 1) pc_tc_kernel(const __gr
                     else if (mode == BIN_THR)
                         bin_chunk<BIN_THR, kBinStride>(g, row_ok, ri, rp, cg, BN, thr_s, mb, fbv,
                                                       ba);
+                    else if (E.pos_ok)
+                        pos_chunk<kBinStride>(g, row_ok, rp, cg, BN, thr_s, mb, fbv, ba);
                     else
                         bin_chunk<BIN_POS, kBinStride>(g, row_ok, ri, rp, cg, BN, thr_s, mb, fbv,
                                                       ba);
