@@ -397,7 +397,7 @@ __device__ __forceinline__ void epi_sync(int nthreads)
     asm volatile("bar.sync 1, %0;" ::"r"(nthreads) : "memory");
 }
 
-// Epilogue barrier that also ANDs a flag over the 128 epilogue threads, so that every
+// Epilogue barrier that also ANDs a flag over the epilogue threads (128 or 256), so that every
 // thread takes the same branch after a bounded wait.
 __device__ __forceinline__ bool epi_sync_and(bool v, int nthreads)
 {
@@ -1722,7 +1722,7 @@ __global__ void __launch_bounds__(tc_threads(BN, EW), 1) pc_tc_kernel(const __gr
         if (ok) flush_q();
     } else {
         // ======================= epilogue =======================
-        const int et = threadIdx.x - 64;          // 0..127
+        const int et = threadIdx.x - 64;          // 0 .. kEpiThreads - 1
         const int q4 = warp & 3;                  // TMEM lane quarter of this warp
         const int r = q4 * 32 + lane;             // accumulator row = tile row
         const int ew = warp - 2;                  // epilogue warp 0..7
