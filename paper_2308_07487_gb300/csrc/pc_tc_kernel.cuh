@@ -128,7 +128,8 @@ __device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity)
 // same test: the tcgen05 fences around the arrive and the wait order the tensor-memory
 // accesses, and TMA and MMA completions are counted by the barrier itself; a cluster-scope
 // acquire in every wait measured 30 % slower.)  Inlined: as a call its saved registers were
-// spilled around every wait of every role; 48^3 glass BF16 94.0 -> 84.1 ms, 32^3 glass
+// spilled around every wait of every role; 48^3 glass BF16 94.0 -> 84.1 ms (86.0 since the phase
+// product has a conversion barrier per accumulator), 32^3 glass
 // split-BF16 19.3 -> 18.8 ms.
 __device__ __forceinline__ bool mbar_wait_for(uint32_t bar, uint32_t parity, int *err, int code,
                                           unsigned long long limit_ns)
